@@ -98,10 +98,11 @@ k_project_grad(const double2 *__restrict__ x, size_t n3, const int *at_cnt,
 __global__ void __launch_bounds__(256)
 k_project_grad_df(const double2 *__restrict__ x, size_t n3, const int *__restrict__ at_cnt,
                   const uint4 *__restrict__ at_rec, const float4 *__restrict__ at_w, int cap,
-                  double h3, double h_kb, int n_orb_pad, double2 *c, double2 *hc, double2 *dc) {
+                  double h3, double h_kb, int n_orb_pad, int split, GatherScratch gs, double2 *c,
+                  double2 *hc, double2 *dc) {
   constexpr int BO = 2, EU = 2;
-  __shared__ double red[8 * 8 * BO];
-  const int J = blockIdx.x, blk = blockIdx.y;
+  __shared__ double red[8 * 8 * BO], res[8 * BO];
+  const int J = blockIdx.x / split, rank = blockIdx.x % split, blk = blockIdx.y;
   const int cnt = at_cnt[J];
   const double2 *xb = x + (size_t)blk * n3 * BO;
   const uint4 *rec = at_rec + (size_t)J * cap;
@@ -109,7 +110,7 @@ k_project_grad_df(const double2 *__restrict__ x, size_t n3, const int *__restric
   float2 ah[4 * BO], al[4 * BO];     // [orbital][c, dc_x, dc_y, dc_z]
 #pragma unroll
   for (int k = 0; k < 4 * BO; ++k) ah[k] = al[k] = make_float2(0.f, 0.f);
-  for (int e0 = threadIdx.x; e0 < cnt; e0 += EU * 256) {
+  for (int e0 = rank * EU * 256 + threadIdx.x; e0 < cnt; e0 += split * EU * 256) {
     uint4 r[EU];
     float4 w0[EU], w1[EU];
 #pragma unroll
@@ -143,16 +144,15 @@ k_project_grad_df(const double2 *__restrict__ x, size_t n3, const int *__restric
     acc[2 * k] = __dadd_rn(df_widen(ah[k].x), df_widen(al[k].x));
     acc[2 * k + 1] = __dadd_rn(df_widen(ah[k].y), df_widen(al[k].y));
   }
-  emd_block_sum<8 * BO>(acc, red);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int j = 0; j < BO; ++j) {
-      const size_t o = (size_t)J * n_orb_pad + (size_t)blk * BO + j;
-      c[o] = make_double2(h3 * acc[8 * j], h3 * acc[8 * j + 1]);
-      hc[o] = make_double2(h_kb * h3 * acc[8 * j], h_kb * h3 * acc[8 * j + 1]);
-      for (int a = 0; a < 3; ++a)
-        dc[3 * o + a] = make_double2(h3 * acc[8 * j + 2 + 2 * a], h3 * acc[8 * j + 3 + 2 * a]);
-    }
+  if (!emd_split_sum<8 * BO>(acc, red, res, gs, J * (int)gridDim.y + blk, rank, split)) return;
+  if (threadIdx.x < BO) {
+    const int j = threadIdx.x;
+    const size_t o = (size_t)J * n_orb_pad + (size_t)blk * BO + j;
+    const double *r = res + 8 * j;
+    c[o] = make_double2(h3 * r[0], h3 * r[1]);
+    hc[o] = make_double2(h_kb * h3 * r[0], h_kb * h3 * r[1]);
+    for (int a = 0; a < 3; ++a)
+      dc[3 * o + a] = make_double2(h3 * r[2 + 2 * a], h3 * r[3 + 2 * a]);
   }
 }
 
@@ -258,10 +258,12 @@ void emd_adj_project_grad(const OrbLayout &o, const TableSet &t, int n_atoms,
   switch (o.bo) {
     case 1: k_project_grad<1><<<grid, 256, 0, st>>>(x, (size_t)o.n3, t.at_cnt, t.at_pt, t.at_p, t.at_d, t.cap, h3, h_kb, inv_rc2, o.n_orb_pad, c, hc, dc); break;
     case 2:
-      if (t.at_rec)
-        k_project_grad_df<<<grid, 256, 0, st>>>(x, (size_t)o.n3, t.at_cnt, t.at_rec, t.at_w,
-                                                t.cap, h3, h_kb, o.n_orb_pad, c, hc, dc);
-      else
+      if (t.at_rec) {
+        const int split = emd_gather_split(n_atoms * o.n_blk, t.cap);
+        k_project_grad_df<<<dim3(n_atoms * split, o.n_blk), 256, 0, st>>>(
+            x, (size_t)o.n3, t.at_cnt, t.at_rec, t.at_w, t.cap, h3, h_kb, o.n_orb_pad, split,
+            o.gs, c, hc, dc);
+      } else
         k_project_grad<2><<<grid, 256, 0, st>>>(x, (size_t)o.n3, t.at_cnt, t.at_pt, t.at_p, t.at_d, t.cap, h3, h_kb, inv_rc2, o.n_orb_pad, c, hc, dc);
       break;
     case 4: k_project_grad<4><<<grid, 256, 0, st>>>(x, (size_t)o.n3, t.at_cnt, t.at_pt, t.at_p, t.at_d, t.cap, h3, h_kb, inv_rc2, o.n_orb_pad, c, hc, dc); break;

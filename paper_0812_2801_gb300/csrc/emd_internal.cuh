@@ -270,6 +270,84 @@ __device__ __forceinline__ void emd_block_sum(double (&v)[NV], double *smem) {
   __syncthreads();
 }
 
+// Scratch of the atom-major gathers that split an atom's entries over several
+// CTAs: NV <= 16 partial sums per CTA and one arrival counter per (projector,
+// orbital block); the counters are zero between launches.  Launches that use
+// one system's scratch are ordered (one stream at a time).
+constexpr int kGatherMaxCtas = 152 * 12 * 2;      // with a split, pairs x split stays below
+struct GatherScratch {
+  double *part = nullptr;                         // [kGatherMaxCtas][16]
+  int *arrived = nullptr;                         // [kGatherMaxCtas / 2]
+};
+// CTAs of 256 threads per (projector, orbital block): one when the pairs fill
+// the GPU, else 2, 4 or 8 that share the atom's entries.  Aims at 12 CTAs per
+// SM and at least one full round of the loop (1024 entries; about half of a
+// table's capacity, a cube around the sphere, is used) per CTA.
+inline int emd_gather_split(int pairs, int cap) {
+  int s = 1;
+  while (s < 8 && pairs * s < kGatherMaxCtas / 2 && cap / 2 >= 1024 * 2 * s) s *= 2;
+  return s;
+}
+
+// Sum of NV (a power of two <= 16) doubles per thread over the 256 threads of
+// `split` CTAs, in an order fixed by the launch shape.  FP64 adds are the cost
+// (one warp instruction per 16 SM cycles), so a warp halves the values it
+// holds at each of its first exchanges instead of carrying all of them
+// through five: 6 adds instead of 20 for NV = 4, 16 instead of 80 for NV =
+// 16.  Then NV threads add the warps in order; the CTA that arrives last at
+// the pair's counter adds the CTAs' sums in rank order and clears the counter.
+// True in that CTA, with the sums in res[0..NV) for every thread of it.
+template <int NV>
+__device__ __forceinline__ bool emd_split_sum(double (&v)[NV], double *smem, double *res,
+                                              const GatherScratch &g, int pair, int rank,
+                                              int split) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int held = NV, o = 16;
+#pragma unroll
+  for (; held > 1; held >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < NV / 2; ++k)
+      if (k < held / 2) {
+        const double keep = up ? v[k + held / 2] : v[k];
+        const double send = up ? v[k] : v[k + held / 2];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  constexpr int PER = 32 / NV;           // lanes that end with the same value
+  if (lane % PER == 0) smem[warp * NV + lane / PER] = v[0];
+  __syncthreads();
+  double a = 0.0;
+  if (threadIdx.x < NV) {
+#pragma unroll
+    for (int w = 0; w < 8; ++w) a += smem[w * NV + threadIdx.x];
+    if (split == 1) res[threadIdx.x] = a;
+    else g.part[((size_t)pair * split + rank) * NV + threadIdx.x] = a;
+  }
+  if (split == 1) {
+    __syncthreads();
+    return true;
+  }
+  __threadfence();
+  __syncthreads();
+  __shared__ int s_last;
+  if (threadIdx.x == 0) s_last = atomicAdd(g.arrived + pair, 1) == split - 1;
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  if (threadIdx.x < NV) {
+    a = 0.0;
+    for (int r = 0; r < split; ++r)
+      a += __ldcg(g.part + ((size_t)pair * split + r) * NV + threadIdx.x);
+    res[threadIdx.x] = a;
+  }
+  if (threadIdx.x == 0) g.arrived[pair] = 0;
+  __syncthreads();
+  return true;
+}
+
 // ---------------------------------------------------------------------------
 // Launchers (defined in the .cu files).  All take the stream to issue on.
 // ---------------------------------------------------------------------------
@@ -392,6 +470,7 @@ struct OrbLayout {
   // the same stencil as integers over a common denominator: c_k = num_k / den
   // (the double-float FP64 stage accumulates with these, exact in FP32)
   double num[EMD_MAX_HALF_ORDER + 1], den;
+  GatherScratch gs;    // complex128, bo = 2
 };
 void emd_launch_stage(const OrbLayout &o, const StageArgs &a, cudaStream_t st);
 void emd_launch_project(const OrbLayout &o, const TableSet &t, int n_atoms,

@@ -1660,11 +1660,12 @@ k_stage_df(const double2 *__restrict__ u_in, const double2 *__restrict__ psi0,
 __global__ void __launch_bounds__(256)
 k_project_df(const double2 *__restrict__ u, size_t n3, const int *__restrict__ at_cnt,
              const uint4 *__restrict__ at_rec, int cap, int nch, double h3, double3 hl,
-             int n_orb_pad, double2 *c, double2 *hc) {
+             int n_orb_pad, int split, GatherScratch gs, double2 *c, double2 *hc) {
   constexpr int BO = 2;
-  __shared__ double red[8 * 2 * BO];
-  // one CTA per (projector P = J nch + k, block): atom J's entries, channel k
-  const int P = blockIdx.x, blk = blockIdx.y;
+  __shared__ double red[8 * 2 * BO], res[2 * BO];
+  // `split` CTAs per (projector P = J nch + k, block): atom
+  // J's entries, channel k, dealt out in rounds of DF_EU x 256
+  const int P = blockIdx.x / split, rank = blockIdx.x % split, blk = blockIdx.y;
   const int cnt = at_cnt[P / nch];
   const int l = emd_channel_l(P % nch);
   const double h_kb = l == 0 ? hl.x : l == 1 ? hl.y : hl.z;
@@ -1673,7 +1674,7 @@ k_project_df(const double2 *__restrict__ u, size_t n3, const int *__restrict__ a
   float2 ah[BO], al[BO];
 #pragma unroll
   for (int j = 0; j < BO; ++j) ah[j] = al[j] = make_float2(0.f, 0.f);
-  for (int e0 = threadIdx.x; e0 < cnt; e0 += DF_EU * 256) {
+  for (int e0 = rank * DF_EU * 256 + threadIdx.x; e0 < cnt; e0 += split * DF_EU * 256) {
     uint4 r[DF_EU];
 #pragma unroll
     for (int v = 0; v < DF_EU; ++v)       // past the end: point 0, p = 0 (adds zero)
@@ -1698,15 +1699,13 @@ k_project_df(const double2 *__restrict__ u, size_t n3, const int *__restrict__ a
     acc[2 * j] = __dadd_rn(df_widen(ah[j].x), df_widen(al[j].x));
     acc[2 * j + 1] = __dadd_rn(df_widen(ah[j].y), df_widen(al[j].y));
   }
-  emd_block_sum<2 * BO>(acc, red);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int j = 0; j < BO; ++j) {
-      const size_t o = (size_t)P * n_orb_pad + (size_t)blk * BO + j;
-      const double re = h3 * acc[2 * j], im = h3 * acc[2 * j + 1];
-      c[o] = make_double2(re, im);
-      hc[o] = make_double2(h_kb * re, h_kb * im);
-    }
+  if (!emd_split_sum<2 * BO>(acc, red, res, gs, P * (int)gridDim.y + blk, rank, split)) return;
+  if (threadIdx.x < BO) {
+    const int j = threadIdx.x;
+    const size_t o = (size_t)P * n_orb_pad + (size_t)blk * BO + j;
+    const double re = h3 * res[2 * j], im = h3 * res[2 * j + 1];
+    c[o] = make_double2(re, im);
+    hc[o] = make_double2(h_kb * re, h_kb * im);
   }
 }
 
@@ -1717,10 +1716,11 @@ __global__ void __launch_bounds__(256)
 k_nl_force_df(const double2 *__restrict__ u, size_t n3, int n_blk,
               const int *__restrict__ at_cnt, const uint4 *__restrict__ at_rec,
               const float4 *__restrict__ at_w, int cap, int nch, const double2 *__restrict__ c,
-              int n_orb_pad, int n_orb, double h3, double3 coef3, double *part) {
+              int n_orb_pad, int n_orb, int split, GatherScratch gs, double h3, double3 coef3,
+              double *part) {
   constexpr int BO = 2, EU = DF_EU;
-  __shared__ double red[8 * 6 * BO];
-  const int P = blockIdx.x, blk = blockIdx.y;
+  __shared__ double red[8 * 16], res[16];
+  const int P = blockIdx.x / split, rank = blockIdx.x % split, blk = blockIdx.y;
   const int cnt = at_cnt[P / nch];
   const int l = emd_channel_l(P % nch);
   const double coef = l == 0 ? coef3.x : l == 1 ? coef3.y : coef3.z;
@@ -1730,7 +1730,7 @@ k_nl_force_df(const double2 *__restrict__ u, size_t n3, int n_blk,
   float2 ah[3 * BO], al[3 * BO];      // [orbital][axis] complex moments
 #pragma unroll
   for (int k = 0; k < 3 * BO; ++k) ah[k] = al[k] = make_float2(0.f, 0.f);
-  for (int e0 = threadIdx.x; e0 < cnt; e0 += EU * 256) {
+  for (int e0 = rank * EU * 256 + threadIdx.x; e0 < cnt; e0 += split * EU * 256) {
     int pt[EU];
     float4 w0[EU], w1[EU];
 #pragma unroll
@@ -1756,7 +1756,7 @@ k_nl_force_df(const double2 *__restrict__ u, size_t n3, int n_blk,
         dfp_add_prod(ah[3 * j + 2], al[3 * j + 2], w1[v].x, w1[v].y, f4hi(xs), f4lo(xs));
       }
   }
-  double acc[6 * BO];
+  double acc[16];                     // 6 BO moments, the rest zero
 #pragma unroll
   for (int j = 0; j < BO; ++j)
 #pragma unroll
@@ -1764,20 +1764,20 @@ k_nl_force_df(const double2 *__restrict__ u, size_t n3, int n_blk,
       acc[6 * j + 2 * a] = __dadd_rn(df_widen(ah[3 * j + a].x), df_widen(al[3 * j + a].x));
       acc[6 * j + 2 * a + 1] = __dadd_rn(df_widen(ah[3 * j + a].y), df_widen(al[3 * j + a].y));
     }
-  emd_block_sum<6 * BO>(acc, red);
-  if (threadIdx.x == 0) {
-    double f[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int k = 6 * BO; k < 16; ++k) acc[k] = 0.0;
+  if (!emd_split_sum<16>(acc, red, res, gs, P * (int)gridDim.y + blk, rank, split)) return;
+  if (threadIdx.x < 3) {
+    const int a = threadIdx.x;
+    double f = 0.0;
     for (int j = 0; j < BO; ++j) {
       const int A = blk * BO + j;
       if (A >= n_orb) continue;
       const double2 cj = c[(size_t)P * n_orb_pad + A];
-      for (int a = 0; a < 3; ++a) {
-        const double dr = h3 * acc[6 * j + 2 * a], di = h3 * acc[6 * j + 2 * a + 1];
-        f[a] += cj.x * dr + cj.y * di;   // Re(conj(c) dc)
-      }
+      const double dr = h3 * res[6 * j + 2 * a], di = h3 * res[6 * j + 2 * a + 1];
+      f += cj.x * dr + cj.y * di;   // Re(conj(c) dc)
     }
-    for (int a = 0; a < 3; ++a)
-      part[((size_t)P * n_blk + blk) * 3 + a] = coef * f[a];
+    part[((size_t)P * n_blk + blk) * 3 + a] = coef * f;
   }
 }
 
@@ -2053,11 +2053,12 @@ void project_t(const OrbLayout &o, const TableSet &t, int n_atoms,
                cudaStream_t st) {
   typedef typename cplx<T>::type V;
   dim3 grid(n_atoms, o.n_blk);
-  if (sizeof(T) == 8 && BO == 2 && t.at_rec)   // one CTA per projector
-    k_project_df<<<dim3(n_atoms * o.nch, o.n_blk), 256, 0, st>>>(
+  if (sizeof(T) == 8 && BO == 2 && t.at_rec) {   // `split` CTAs per (projector, block)
+    const int split = emd_gather_split(n_atoms * o.nch * o.n_blk, t.cap);
+    k_project_df<<<dim3(n_atoms * o.nch * split, o.n_blk), 256, 0, st>>>(
         (const double2 *)u, (size_t)o.n3, t.at_cnt, t.at_rec, t.cap, o.nch, h3,
-        make_double3(h_kb, o.hl[1], o.hl[2]), o.n_orb_pad, c, (double2 *)hc);
-  else
+        make_double3(h_kb, o.hl[1], o.hl[2]), o.n_orb_pad, split, o.gs, c, (double2 *)hc);
+  } else
     k_project<T, BO><<<grid, 256, 0, st>>>((const V *)u, (size_t)o.n3, t.at_cnt,
                                            t.at_pt, t.at_p, t.cap, h3, h_kb,
                                            o.n_orb_pad, c, (V *)hc);
@@ -2106,9 +2107,10 @@ void nlf_t(const OrbLayout &o, const TableSet &t, int n_atoms, const void *u,
   if (sizeof(T) == 8 && BO == 2 && t.at_rec) {
     // the s channel keeps coef = -2 h_kb occ as given
     const double3 coef3 = make_double3(coef, coef_unit * o.hl[1], coef_unit * o.hl[2]);
-    k_nl_force_df<<<dim3(n_atoms * o.nch, o.n_blk), 256, 0, st>>>(
+    const int split = emd_gather_split(n_atoms * o.nch * o.n_blk, t.cap);
+    k_nl_force_df<<<dim3(n_atoms * o.nch * split, o.n_blk), 256, 0, st>>>(
         (const double2 *)u, (size_t)o.n3, o.n_blk, t.at_cnt, t.at_rec, t.at_w, t.cap, o.nch, c,
-        o.n_orb_pad, o.n_orb, h3, coef3, part);
+        o.n_orb_pad, o.n_orb, split, o.gs, h3, coef3, part);
   } else
     k_nl_force<T, BO><<<grid, 256, 0, st>>>((const V *)u, (size_t)o.n3, o.n_blk,
                                             t.at_cnt, t.at_pt, t.at_p, t.at_d,
