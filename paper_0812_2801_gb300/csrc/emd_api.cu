@@ -132,6 +132,7 @@ struct emd_system {
   double *veff1 = nullptr, *veff2 = nullptr;
   float *veff1f = nullptr, *veff2f = nullptr;
   float4 *veff1d = nullptr, *veff2d = nullptr;   // complex64: (w_0 + v_eff) x4
+  float2 *veff1s = nullptr, *veff2s = nullptr;   // complex128, bo = 2: split diagonal
   double *hist[3] = {nullptr, nullptr, nullptr};
   int hist_len = 0;
   double *rho = nullptr, *v_h = nullptr, *v_xc = nullptr, *eps_xc = nullptr;
@@ -276,14 +277,15 @@ int table_pipe(emd_system *s) {
 
 void negate_grid(double *v, int n3, cudaStream_t st);
 
-void project(emd_system *s, const void *u, int set, cudaStream_t st) {
+// u_split: u is a split set (see StageArgs), complex128 with bo = 2 only
+void project(emd_system *s, const void *u, int set, cudaStream_t st, bool u_split = false) {
   if (s->o.prec == EMD_FP32_ORBITALS)
     emd_launch_project_tile(s->o, s->ts[set], s->n_atoms, u,
                             s->g.h * s->g.h * s->g.h, s->sp.h_kb, s->c, s->hc,
                             s->proj_part, st);
   else if (s->proj_atom_major || s->sp.nch > 1)
     emd_launch_project(s->o, s->ts[set], s->n_atoms, u, s->g.h * s->g.h * s->g.h,
-                       s->sp.h_kb, s->c, s->hc, st);
+                       s->sp.h_kb, s->c, s->hc, st, u_split);
   else
     emd_launch_project_pm(s->o, s->ts[set], s->n_atoms, u,
                           s->g.h * s->g.h * s->g.h, s->sp.h_kb, s->c, s->hc,
@@ -292,13 +294,16 @@ void project(emd_system *s, const void *u, int set, cudaStream_t st) {
 void project(emd_system *s, const void *u, int set) { project(s, u, set, s->st); }
 
 void stage(emd_system *s, const void *u_in, const void *psi0, void *u_out,
-           int set, int which_veff, double a) {
+           int set, int which_veff, double a, int in_split = 0, int out_split = 0) {
   StageArgs a_;
+  a_.in_split = in_split;
+  a_.out_split = out_split;
   a_.u_in = u_in;
   a_.psi0 = psi0;
   a_.u_out = u_out;
   if (s->o.prec == EMD_FP64) {
     a_.v_eff = which_veff == 1 ? (const void *)s->veff1 : (const void *)s->veff2;
+    a_.v_diag = which_veff == 1 ? (const void *)s->veff1s : (const void *)s->veff2s;
   } else {
     a_.v_eff = which_veff == 1 ? (const void *)s->veff1f : (const void *)s->veff2f;
     a_.v_diag = which_veff == 1 ? (const void *)s->veff1d : (const void *)s->veff2d;
@@ -327,16 +332,20 @@ void stage(emd_system *s, const void *u_in, const void *psi0, void *u_out,
 }
 
 // One exponential T4(-i tau H) psi0 -> out, H given by (set, veff).
-// Requires hc to hold the projections of psi0 at `set` on entry.
+// Requires hc to hold the projections of psi0 at `set` on entry, and the
+// split diagonal of the potential if the system has one.  The double-float
+// stage keeps the three intermediate sets as split values.
 void exponential(emd_system *s, void *psi0, void *w1, void *out, int set,
                  int which_veff, double tau) {
-  stage(s, psi0, psi0, w1, set, which_veff, tau / 4.0);
-  project(s, w1, set);
-  stage(s, w1, psi0, out, set, which_veff, tau / 3.0);
-  project(s, out, set);
-  stage(s, out, psi0, w1, set, which_veff, tau / 2.0);
-  project(s, w1, set);
-  stage(s, w1, psi0, out, set, which_veff, tau);
+  const int sp = s->veff1s && s->o.stage_variant != 1 &&
+                 (s->proj_atom_major || s->sp.nch > 1) && emd_stage_df_splits(s->o);
+  stage(s, psi0, psi0, w1, set, which_veff, tau / 4.0, 0, sp);
+  project(s, w1, set, s->st, sp);
+  stage(s, w1, psi0, out, set, which_veff, tau / 3.0, sp, sp);
+  project(s, out, set, s->st, sp);
+  stage(s, out, psi0, w1, set, which_veff, tau / 2.0, sp, sp);
+  project(s, w1, set, s->st, sp);
+  stage(s, w1, psi0, out, set, which_veff, tau, sp, 0);
 }
 
 // rho, v_H, v_xc of psi into hist slot `slot`.
@@ -608,6 +617,10 @@ int emd_init_system(const emd_config *cfg, emd_system **out) {
     TRY(A((void **)&s->veff2f, n3 * 4));
     TRY(A((void **)&s->veff1d, n3 * 16));
     TRY(A((void **)&s->veff2d, n3 * 16));
+  }
+  if (c.precision == EMD_FP64 && o.bo == 2) {
+    TRY(A((void **)&s->veff1s, n3 * 8));
+    TRY(A((void **)&s->veff2s, n3 * 8));
   }
   for (int k = 0; k < 3; ++k) TRY(A((void **)&s->hist[k], n3 * 8));
   TRY(A((void **)&s->rho, n3 * 8));
@@ -991,14 +1004,16 @@ int step_once(emd_system *s, double dt, double mu, double e) {
     if (r) return r;
     negate_grid(s->ts[nw].v_loc, s->g.n3, s->tst);
     emd_launch_veff(s->g, s->ts[nw].v_loc, s->hist, s->hist_len, e, s->veff2,
-                    s->veff2f, s->tst, s->veff2d, s->o.w[0]);
+                    s->veff2f, s->tst, s->veff2d, s->o.w[0], s->veff2s, s->o.dv_scale(),
+                    s->o.dv_shift());
     CK(cudaEventRecord(s->tev[1], s->tst));
   } else {
     emd_launch_veff(s->g, s->ts[nw].v_loc, s->hist, s->hist_len, e, s->veff2,
-                    s->veff2f, s->st, s->veff2d, s->o.w[0]);
+                    s->veff2f, s->st, s->veff2d, s->o.w[0], s->veff2s, s->o.dv_scale(),
+                    s->o.dv_shift());
   }
   emd_launch_veff(s->g, s->ts[cur].v_loc, s->hist, 1, e, s->veff1, s->veff1f,
-                  s->st, s->veff1d, s->o.w[0]);
+                  s->st, s->veff1d, s->o.w[0], s->veff1s, s->o.dv_scale(), s->o.dv_shift());
   if (!s->c_valid) project(s, s->psi, cur);
   // exponential 1: psi -> ub with H(t)
   exponential(s, s->psi, s->ua, s->ub, cur, 1, tau);

@@ -222,6 +222,19 @@ __device__ __forceinline__ float4 df_split2(double2 v) {
 __device__ __forceinline__ float2 f4hi(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 f4lo(float4 v) { return make_float2(v.z, v.w); }
 
+// ---- per-thread asynchronous copies to shared memory ------------------------
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+template <int N> __device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Exact displacement arithmetic.  The support decision d^2 < r^2 is an
 // integer decision taken in FP64 from the same operations, in the same
@@ -397,11 +410,13 @@ void emd_launch_lda(int n3, const double *rho, const double *v_h,
                     double *eps_xc, double *v_xc, double *vhxc,
                     cudaStream_t st);
 // v_eff = v_loc + extrapolated v_Hxc + field term (FP64 and, if v_eff_f,
-// FP32); if v_diag, also (d, d, d, d) with d = w0 + v_eff in FP32
+// FP32); if v_diag, also (d, d, d, d) with d = w0 + v_eff in FP32; if
+// v_split, dv_shift + dv_scale v_eff split into (hi, lo)
 void emd_launch_veff(const GridInfo &g, const double *v_loc,
                      const double *const *hist, int hist_len, double field,
                      double *v_eff, float *v_eff_f, cudaStream_t st,
-                     float4 *v_diag = nullptr, double w0 = 0.0);
+                     float4 *v_diag = nullptr, double w0 = 0.0, float2 *v_split = nullptr,
+                     double dv_scale = 0.0, double dv_shift = 0.0);
 // partials[b] = block sums of (a - c)(b + d); c, d, b may be NULL
 void emd_launch_dot_partials(int n3, const double *a, const double *b,
                              const double *c, const double *d,
@@ -450,12 +465,17 @@ struct StageArgs {
   const void *psi0;
   void *u_out;
   const void *v_eff;       // double* (FP64) or float* (FP32)
-  const void *v_diag = nullptr;   // FP32: float4 (d, d, d, d), d = w_0 + v_eff
+  const void *v_diag = nullptr;   // FP32: float4 (d, d, d, d), d = w_0 + v_eff;
+                                  // FP64, bo = 2: float2, the split diagonal
   const TableSet *tab;
   const void *hc;          // [n_atoms][n_orb_pad] h_kb*c in orbital precision
   double a;                // tau / k ; u_out = psi0 + (-i a) H u_in
   int apply_only;          // 1: u_out = H u_in (psi0 unused)
   int *err = nullptr;      // device error bits (EMD_ERRBIT_*), may be NULL
+  // complex128, bo = 2: u_in / u_out as split double-float values (float4 (re
+  // hi, im hi, re lo, im lo) in place of each double2); in_split needs v_diag,
+  // the split diagonal (float2 per point)
+  int in_split = 0, out_split = 0;
 };
 struct OrbLayout {
   int n, n3, bo, n_blk, n_orb, n_orb_pad, prec, half_order, n_atoms;
@@ -471,11 +491,17 @@ struct OrbLayout {
   // (the double-float FP64 stage accumulates with these, exact in FP32)
   double num[EMD_MAX_HALF_ORDER + 1], den;
   GatherScratch gs;    // complex128, bo = 2
+  // the double-float stage's diagonal dv = dv_shift + dv_scale v_eff
+  double dv_scale() const { return -2.0 * h * h * den; }
+  double dv_shift() const { return 3.0 * num[0]; }
 };
 void emd_launch_stage(const OrbLayout &o, const StageArgs &a, cudaStream_t st);
+// stage_df.cu: the complex128, bo = 2 stage in double-float arithmetic
+void emd_launch_stage_df(const OrbLayout &o, const StageArgs &a, cudaStream_t st);
+bool emd_stage_df_splits(const OrbLayout &o);   // takes and writes split sets
 void emd_launch_project(const OrbLayout &o, const TableSet &t, int n_atoms,
                         const void *u, double h3, double h_kb, double2 *c,
-                        void *hc, cudaStream_t st);
+                        void *hc, cudaStream_t st, bool u_split = false);
 void emd_launch_density(const OrbLayout &o, const void *u, double occ,
                         double *rho, cudaStream_t st);
 void emd_launch_kinetic_partials(const OrbLayout &o, const void *u,

@@ -136,18 +136,6 @@ k_stage(const typename cplx<T>::type *__restrict__ u_in,
 // rows, so y-neighbours come from a register window (RY + 2M loads for RY
 // outputs) and x-neighbours from shared memory (2M loads per output).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-template <int N> __device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
 template <int BO, int M> struct ZTile {
   static constexpr int NC = 64;                 // orbital columns = threads in x
   static constexpr int TX = NC / BO;            // points per tile in x
@@ -1370,281 +1358,6 @@ k_abs2_sum(const double2 *c, int n, int row, int nch, double3 w, double *out) {
   if (threadIdx.x == 0) *out = acc[0];
 }
 
-// ---------------------------------------------------------------------------
-// FP64 Horner stage in double-float arithmetic (complex128 orbitals, bo = 2).
-// GB300 issues one FP64 warp instruction per 16 SM cycles, and the plain FP64
-// stage spends ~59 FP64 instructions per update.  Here every value of a
-// staged plane is split once into two floats, x = hi + lo (hi: the top 24
-// significand bits, lo: the rest rounded to 24 bits; 48 bits in all), by
-// integer operations on its bits, and the stencil runs on the FP32 pipes:
-// products by the integer FD numerators num_k (exact in FP32) through
-// TwoProduct with an FMA, sums through Knuth's TwoSum, the rounding errors
-// gathered in the low word.  The accumulated K = dv u + sum_k num_k S_k,
-// dv = 3 num_0 - 2 h^2 den v_eff, gives H u = -K / (2 h^2 den) + V_nl u; only
-// the conversion of H u back to double and the Taylor update use FP64
-// instructions (four per update).  The tile marches through z like the
-// complex64 column kernels; each thread owns one orbital of one point, the
-// z-direction accumulates in a (2M+1)-slot shift register, and planes are
-// staged through registers (load, split, store) one plane ahead.
-// ---------------------------------------------------------------------------
-struct DFWeights {
-  float num[EMD_MAX_HALF_ORDER + 1];   // FD numerators, exact in FP32
-  float sk_hi, sk_lo;                  // -1 / (2 h^2 den) as double-float
-  double dvs, dv0;                     // dv = dv0 + dvs v_eff
-};
-
-template <int M> struct DFTile {
-  static constexpr int BO = 2;
-  static constexpr int NC = 64;                 // orbital columns = threads in x
-  static constexpr int TX = NC / BO;            // points per tile row
-  static constexpr int NT = 512;
-  static constexpr int TY = NT / NC;            // rows, one per thread row
-  static constexpr int SW = TX + 2 * M, SH = TY + 2 * M;
-  static constexpr int NCH = SH * SW * BO;      // complex values per staged plane
-  static constexpr int CPT = (NCH + NT - 1) / NT;
-  static constexpr int NV = TX * TY;            // tile points
-  static constexpr int NS = 2 * M + 1;          // shift-register slots
-  // raw slot (3, cp.async, two planes ahead): plane as complex128 | v_eff of
-  // the tile points | records and psi0 of the output plane completed by it
-  static constexpr int RU = NCH * 16, RV = NV * 8, RQ = NV * 48, RP = NV * BO * 16;
-  static constexpr int RSLOT = RU + RV + RQ + RP;
-  // split slot (2): plane as double-float complex | dv of the tile points
-  static constexpr int DU = NCH * 16, DD = NV * 8;
-  static constexpr int DSLOT = DU + DD;
-  static constexpr size_t SMEM_FIXED = 3 * (size_t)RSLOT + 2 * (size_t)DSLOT;
-};
-
-// MP: several projectors per atom (the pre-split records past the first four
-// are read with four in flight); a separate instantiation keeps the
-// s-projector kernel's registers as they were
-template <int M, bool HCS, bool MP>
-__global__ void __launch_bounds__(512, 1)
-k_stage_df(const double2 *__restrict__ u_in, const double2 *__restrict__ psi0,
-           double2 *__restrict__ u_out, const double *__restrict__ v_eff,
-           const int4 *__restrict__ pt4d, const int *__restrict__ pt_J,
-           const double *__restrict__ pt_p, const int4 *__restrict__ pt_rec,
-           const double2 *__restrict__ hc, int n,
-           int ntx, int zc, int n_orb_pad, int n_atoms, double a, int apply_only,
-           DFWeights W) {
-  typedef DFTile<M> Z;
-  constexpr int BO = Z::BO, NS = Z::NS, SW = Z::SW, NT = Z::NT;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned char *dfbase = smraw + 3 * Z::RSLOT;
-  float4 *hcs = reinterpret_cast<float4 *>(smraw + Z::SMEM_FIXED);
-  const int tid = threadIdx.x;
-  const int col = tid % Z::NC, tyr = tid / Z::NC;
-  const int xl = col / BO, j = col % BO;
-  const int tx0 = (blockIdx.x % ntx) * Z::TX, ty0 = (blockIdx.x / ntx) * Z::TY;
-  const int z0 = blockIdx.y * zc;
-  const int zcount = min(zc, n - z0);
-  const int total = zcount + 2 * M;
-  const int n2 = n * n;
-  const size_t n3 = (size_t)n2 * n;
-  const size_t boff = (size_t)blockIdx.z * n3 * BO;
-  const double2 *ub = u_in + boff;
-  const double2 *pb = psi0 + boff;
-  double2 *ob = u_out + boff;
-  const int x = tx0 + xl, y = ty0 + tyr;
-  const bool valid = x < n && y < n;
-  const size_t pxy = (size_t)min(y, n - 1) * n + min(x, n - 1);
-
-  // staging map of the plane values: source index within a plane, -1 = none
-  int src[Z::CPT];
-#pragma unroll
-  for (int i = 0; i < Z::CPT; ++i) {
-    const int q = tid + i * NT;
-    src[i] = -1;
-    if (q < Z::NCH) {
-      const int jj = q % BO, pnt = q / BO;
-      const int c = pnt % SW, rr = pnt / SW;
-      const int xx = (tx0 - M + c + 2 * n) % n;
-      const int yy = (ty0 - M + rr + 2 * n) % n;
-      src[i] = (yy * n + xx) * BO + jj;
-    }
-  }
-  // tile point of this thread in the per-point stagings (v_eff, records)
-  const int vp = tid < Z::NV ? min(ty0 + tid / Z::TX, n - 1) * n + min(tx0 + tid % Z::TX, n - 1)
-                             : -1;
-  if (HCS) {
-    for (int i = tid; i < n_atoms * BO; i += NT)
-      hcs[i] = df_split2(hc[(size_t)(i / BO) * n_orb_pad + (size_t)blockIdx.z * BO + i % BO]);
-  }
-  const unsigned sm0 = (unsigned)__cvta_generic_to_shared(smraw);
-
-  auto issue = [&](int zi) {
-    const unsigned base = sm0 + (zi % 3) * Z::RSLOT;
-    int zz = z0 - M + zi;
-    zz += zz < 0 ? n : 0;
-    zz -= zz >= n ? n : 0;
-    const size_t poff = (size_t)zz * n2;
-#pragma unroll
-    for (int i = 0; i < Z::CPT; ++i)
-      if (src[i] >= 0)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(base + (tid + i * NT) * 16),
-                     "l"(ub + poff * BO + src[i]) : "memory");
-    if (vp >= 0)
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(base + Z::RU + tid * 8),
-                   "l"(v_eff + poff + vp) : "memory");
-    if (zi >= 2 * M && vp >= 0) {
-      const size_t po = (size_t)(z0 + zi - 2 * M) * n2 + vp;
-#pragma unroll
-      for (int k = 0; k < 3; ++k)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(
-                         base + Z::RU + Z::RV + (tid * 3 + k) * 16),
-                     "l"(pt4d + po * 3 + k) : "memory");
-      if (!apply_only) {
-#pragma unroll
-        for (int jj = 0; jj < BO; ++jj)
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(
-                           base + Z::RU + Z::RV + Z::RQ + (tid * BO + jj) * 16),
-                       "l"(pb + po * BO + jj) : "memory");
-      }
-    }
-    cp_async_commit();
-  };
-  // split the raw plane zi into double-float slot zi & 1
-  auto convert = [&](int zi) {
-    const unsigned char *raw = smraw + (zi % 3) * Z::RSLOT;
-    unsigned char *dst = dfbase + (zi & 1) * Z::DSLOT;
-    const double2 *R = reinterpret_cast<const double2 *>(raw);
-    float4 *D = reinterpret_cast<float4 *>(dst);
-#pragma unroll
-    for (int i = 0; i < Z::CPT; ++i)
-      if (src[i] >= 0) D[tid + i * NT] = df_split2(R[tid + i * NT]);
-    if (vp >= 0)
-      reinterpret_cast<float2 *>(dst + Z::DU)[tid] =
-          df_split(__fma_rn(W.dvs, reinterpret_cast<const double *>(raw + Z::RU)[tid], W.dv0));
-  };
-
-  // ah, al [s]: output plane zi - M + s, K as hi = (re, im), lo = (re, im)
-  float2 ah[NS], al[NS];
-#pragma unroll
-  for (int s = 0; s < NS; ++s) ah[s] = al[s] = make_float2(0.f, 0.f);
-  const int ci = ((tyr + M) * SW + xl + M) * BO + j;       // centre, float4 index
-  const int pt = tyr * Z::TX + xl;                         // tile point index
-  const char *hcj = reinterpret_cast<const char *>(hcs + j);
-  const double2 *hcg = hc + (size_t)blockIdx.z * BO + j;
-
-  issue(0);
-  if (total > 1) issue(1);
-  if (total > 1) cp_async_wait<1>();
-  else cp_async_wait<0>();
-  __syncthreads();
-  convert(0);
-  for (int zi = 0; zi < total; ++zi) {
-    // raw plane zi + 1 (issued one iteration ago) is the only group in flight
-    cp_async_wait<0>();
-    // one barrier: raw zi + 1 visible; split zi (converted last iteration)
-    // visible; every thread has finished iteration zi - 1, so split slot
-    // (zi + 1) & 1 and raw slot (zi + 2) % 3 are free
-    __syncthreads();
-    if (zi + 2 < total) issue(zi + 2);
-    if (zi + 1 < total) convert(zi + 1);
-    const unsigned char *base = dfbase + (zi & 1) * Z::DSLOT;
-    const float4 *P = reinterpret_cast<const float4 *>(base) + ci;
-    const float2 d = reinterpret_cast<const float2 *>(base + Z::DU)[pt];
-    const float4 c = P[0];
-    const float2 ch = f4hi(c), cl = f4lo(c);
-    // own plane: dv u + the x/y shells
-    dfp_add_prod(ah[M], al[M], d.x, d.y, ch, cl);
-#pragma unroll
-    for (int k = 1; k <= M; ++k) {
-      const float4 v1 = P[k * BO], v2 = P[-k * BO], v3 = P[k * SW * BO], v4 = P[-k * SW * BO];
-      float2 sh = f4hi(v1), sl = f4lo(v1);
-      dfp_add(sh, sl, f4hi(v2), f4lo(v2));
-      dfp_add(sh, sl, f4hi(v3), f4lo(v3));
-      dfp_add(sh, sl, f4hi(v4), f4lo(v4));
-      const float2 w2 = make_float2(W.num[k], W.num[k]);
-      float2 p, pe;
-      dfp_two_prod(w2, sh, p, pe);
-      dfp_add(ah[M], al[M], p, __ffma2_rn(w2, sl, pe));
-    }
-    // z-direction: this plane is neighbour k of output planes zi +- k
-#pragma unroll
-    for (int k = 1; k <= M; ++k) {
-      const float2 w2 = make_float2(W.num[k], W.num[k]);
-      float2 p, pe;
-      dfp_two_prod(w2, ch, p, pe);
-      const float2 q = __ffma2_rn(w2, cl, pe);
-      dfp_add(ah[M + k], al[M + k], p, q);
-      if (zi >= k) dfp_add(ah[M - k], al[M - k], p, q);
-    }
-    if (zi >= 2 * M && valid) {   // output plane z0 + zi - 2M is complete in slot 0
-      const unsigned char *raw = smraw + (zi % 3) * Z::RSLOT;
-      const int4 *Q = reinterpret_cast<const int4 *>(raw + Z::RU + Z::RV) + pt * 3;
-      const int4 q0 = Q[0], q1 = Q[1], q2 = Q[2];
-      float2 hh = make_float2(0.f, 0.f), hl = make_float2(0.f, 0.f);
-      dfp_add_prod(hh, hl, W.sk_hi, W.sk_lo, ah[0], al[0]);
-      // four entries (unused ones have p = 0 and add exactly zero)
-      const int Je[4] = {q0.x & 0xffff, q0.y, q0.z, q0.w};
-      const float ph[4] = {__int_as_float(q1.x), __int_as_float(q1.z), __int_as_float(q2.x),
-                           __int_as_float(q2.z)};
-      const float pl[4] = {__int_as_float(q1.y), __int_as_float(q1.w), __int_as_float(q2.y),
-                           __int_as_float(q2.w)};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float4 h4 = HCS ? *reinterpret_cast<const float4 *>(hcj + Je[e] * (BO * 16))
-                              : df_split2(hcg[(size_t)Je[e] * n_orb_pad]);
-        dfp_add_prod(hh, hl, ph[e], pl[e], f4hi(h4), f4lo(h4));
-      }
-      const int cnt = q0.x >> 16;
-      if (cnt > 4) {
-        const size_t p = (size_t)(z0 + zi - 2 * M) * n2 + pxy;
-        if (MP) {
-          // several projectors per atom: pre-split 16-byte records, four in
-          // flight, summed into four independent pairs (combined in a fixed
-          // order) so that the TwoSum chains overlap
-          float2 xh[4], xl[4];
-#pragma unroll
-          for (int v = 0; v < 4; ++v) xh[v] = xl[v] = make_float2(0.f, 0.f);
-          for (int e = 4; e < cnt; e += 4) {
-            int4 q[4];
-#pragma unroll
-            for (int v = 0; v < 4; ++v)
-              q[v] = e + v < cnt ? __ldg(pt_rec + (size_t)(e + v) * n3 + p) : make_int4(0, 0, 0, 0);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              const float4 h4 = HCS ? *reinterpret_cast<const float4 *>(hcj + q[v].x * (BO * 16))
-                                    : df_split2(hcg[(size_t)q[v].x * n_orb_pad]);
-              dfp_add_prod(xh[v], xl[v], __int_as_float(q[v].y), __int_as_float(q[v].z),
-                           f4hi(h4), f4lo(h4));
-            }
-          }
-#pragma unroll
-          for (int v = 0; v < 4; ++v) dfp_add(hh, hl, xh[v], xl[v]);
-        } else {
-          for (int e = 4; e < cnt; ++e) {
-            const int J = pt_J[(size_t)e * n3 + p];
-            const float2 pv = df_split(pt_p[(size_t)e * n3 + p]);
-            const float4 h4 = HCS ? *reinterpret_cast<const float4 *>(hcj + J * (BO * 16))
-                                  : df_split2(hcg[(size_t)J * n_orb_pad]);
-            dfp_add_prod(hh, hl, pv.x, pv.y, f4hi(h4), f4lo(h4));
-          }
-        }
-      }
-      const double Hr = __dadd_rn(df_widen(hh.x), df_widen(hl.x));
-      const double Hi = __dadd_rn(df_widen(hh.y), df_widen(hl.y));
-      double2 out;
-      if (apply_only) {
-        out = make_double2(Hr, Hi);
-      } else {
-        const double2 sv =
-            reinterpret_cast<const double2 *>(raw + Z::RU + Z::RV + Z::RQ)[pt * BO + j];
-        out.x = __fma_rn(a, Hi, sv.x);
-        out.y = __fma_rn(-a, Hr, sv.y);
-      }
-      ob[((size_t)(z0 + zi - 2 * M) * n2 + pxy) * BO + j] = out;
-    }
-    // shift the register line: output plane zi - M + 1 moves to slot 0
-#pragma unroll
-    for (int s = 0; s < NS - 1; ++s) {
-      ah[s] = ah[s + 1];
-      al[s] = al[s + 1];
-    }
-    ah[NS - 1] = al[NS - 1] = make_float2(0.f, 0.f);
-  }
-}
-
 // complex128 projections and nonlocal-force moments (bo = 2) in double-float
 // arithmetic on the FP32 pipes: the FP64 forms spend 2 (projection) and 8
 // (moments) FP64 instructions per table entry and orbital, which bounds them
@@ -1657,8 +1370,10 @@ k_stage_df(const double2 *__restrict__ u_in, const double2 *__restrict__ psi0,
 // join the fixed-tree FP64 block sum.
 #define DF_EU 4
 
+// IN: u as split values (the stages' intermediate sets)
+template <bool IN>
 __global__ void __launch_bounds__(256)
-k_project_df(const double2 *__restrict__ u, size_t n3, const int *__restrict__ at_cnt,
+k_project_df(const void *__restrict__ u, size_t n3, const int *__restrict__ at_cnt,
              const uint4 *__restrict__ at_rec, int cap, int nch, double h3, double3 hl,
              int n_orb_pad, int split, GatherScratch gs, double2 *c, double2 *hc) {
   constexpr int BO = 2;
@@ -1669,7 +1384,7 @@ k_project_df(const double2 *__restrict__ u, size_t n3, const int *__restrict__ a
   const int cnt = at_cnt[P / nch];
   const int l = emd_channel_l(P % nch);
   const double h_kb = l == 0 ? hl.x : l == 1 ? hl.y : hl.z;
-  const double2 *ub = u + (size_t)blk * n3 * BO;
+  const float4 *ub = static_cast<const float4 *>(u) + (size_t)blk * n3 * BO;   // 16-byte values
   const uint4 *rec = at_rec + (size_t)P * cap;
   float2 ah[BO], al[BO];
 #pragma unroll
@@ -1679,7 +1394,7 @@ k_project_df(const double2 *__restrict__ u, size_t n3, const int *__restrict__ a
 #pragma unroll
     for (int v = 0; v < DF_EU; ++v)       // past the end: point 0, p = 0 (adds zero)
       r[v] = e0 + 256 * v < cnt ? __ldg(rec + e0 + 256 * v) : make_uint4(0u, 0u, 0u, 0u);
-    double2 x[DF_EU][BO];
+    float4 x[DF_EU][BO];
 #pragma unroll
     for (int v = 0; v < DF_EU; ++v)
 #pragma unroll
@@ -1688,7 +1403,7 @@ k_project_df(const double2 *__restrict__ u, size_t n3, const int *__restrict__ a
     for (int v = 0; v < DF_EU; ++v)
 #pragma unroll
       for (int j = 0; j < BO; ++j) {
-        const float4 xs = df_split2(x[v][j]);
+        const float4 xs = IN ? x[v][j] : df_split2(*reinterpret_cast<const double2 *>(&x[v][j]));
         dfp_add_prod(ah[j], al[j], __uint_as_float(r[v].y), __uint_as_float(r[v].z), f4hi(xs),
                      f4lo(xs));
       }
@@ -1982,54 +1697,6 @@ void stage_z_m(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
   }
 }
 
-template <int M, bool HCS, bool MP>
-void stage_df_tt(const OrbLayout &o, const StageArgs &a, size_t smem, cudaStream_t st) {
-  typedef DFTile<M> Z;
-  static bool attr_done = false;
-  if (!attr_done) {
-    cudaFuncSetAttribute(k_stage_df<M, HCS, MP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(Z::SMEM_FIXED + 32768));
-    attr_done = true;
-  }
-  const int ntx = (o.n + Z::TX - 1) / Z::TX, nty = (o.n + Z::TY - 1) / Z::TY;
-  const int zc = stage_zchunk(o, ntx * nty * o.n_blk, 2 * 152);
-  DFWeights W;
-  for (int k = 0; k <= EMD_MAX_HALF_ORDER; ++k) W.num[k] = (float)o.num[k];
-  const double sk = -1.0 / (2.0 * o.h * o.h * o.den);
-  W.sk_hi = (float)sk;
-  W.sk_lo = (float)(sk - (double)W.sk_hi);
-  W.dvs = -2.0 * o.h * o.h * o.den;
-  W.dv0 = 3.0 * o.num[0];
-  dim3 grid(ntx * nty, (o.n + zc - 1) / zc, o.n_blk);
-  k_stage_df<M, HCS, MP><<<grid, Z::NT, smem, st>>>(
-      (const double2 *)a.u_in, (const double2 *)a.psi0, (double2 *)a.u_out,
-      (const double *)a.v_eff, a.tab->pt4d, a.tab->pt_J, a.tab->pt_p, a.tab->pt_rec,
-      (const double2 *)a.hc, o.n, ntx, zc, o.n_orb_pad, o.n_proj, a.a, a.apply_only, W);
-}
-
-template <int M>
-void stage_df_t(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
-  typedef DFTile<M> Z;
-  const int hc_bytes = o.n_proj * Z::BO * (int)sizeof(float4);   // every projector's h c
-  const bool mp = a.tab->pt_rec != nullptr;
-  if (hc_bytes <= 32768) {
-    if (mp) stage_df_tt<M, true, true>(o, a, Z::SMEM_FIXED + hc_bytes, st);
-    else stage_df_tt<M, true, false>(o, a, Z::SMEM_FIXED + hc_bytes, st);
-  } else {
-    if (mp) stage_df_tt<M, false, true>(o, a, Z::SMEM_FIXED, st);
-    else stage_df_tt<M, false, false>(o, a, Z::SMEM_FIXED, st);
-  }
-}
-
-inline void stage_df_m(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
-  switch (o.half_order) {
-    case 1: stage_df_t<1>(o, a, st); break;
-    case 2: stage_df_t<2>(o, a, st); break;
-    case 3: stage_df_t<3>(o, a, st); break;
-    case 4: stage_df_t<4>(o, a, st); break;
-  }
-}
-
 template <typename T, int BO>
 void stage_m(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
   switch (o.half_order) {
@@ -2050,13 +1717,14 @@ void stage_m(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
 template <typename T, int BO>
 void project_t(const OrbLayout &o, const TableSet &t, int n_atoms,
                const void *u, double h3, double h_kb, double2 *c, void *hc,
-               cudaStream_t st) {
+               cudaStream_t st, bool u_split) {
   typedef typename cplx<T>::type V;
   dim3 grid(n_atoms, o.n_blk);
   if (sizeof(T) == 8 && BO == 2 && t.at_rec) {   // `split` CTAs per (projector, block)
     const int split = emd_gather_split(n_atoms * o.nch * o.n_blk, t.cap);
-    k_project_df<<<dim3(n_atoms * o.nch * split, o.n_blk), 256, 0, st>>>(
-        (const double2 *)u, (size_t)o.n3, t.at_cnt, t.at_rec, t.cap, o.nch, h3,
+    auto kernel = u_split ? k_project_df<true> : k_project_df<false>;
+    kernel<<<dim3(n_atoms * o.nch * split, o.n_blk), 256, 0, st>>>(
+        u, (size_t)o.n3, t.at_cnt, t.at_rec, t.cap, o.nch, h3,
         make_double3(h_kb, o.hl[1], o.hl[2]), o.n_orb_pad, split, o.gs, c, (double2 *)hc);
   } else
     k_project<T, BO><<<grid, 256, 0, st>>>((const V *)u, (size_t)o.n3, t.at_cnt,
@@ -2151,7 +1819,7 @@ void emd_launch_stage(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
       case 1: stage_m<double, 1>(o, a, st); break;
       case 2:
         if (o.stage_variant == 1 || !a.tab->pt4d) stage_m<double, 2>(o, a, st);
-        else stage_df_m(o, a, st);
+        else emd_launch_stage_df(o, a, st);
         break;
       case 4: stage_m<double, 4>(o, a, st); break;
     }
@@ -2176,13 +1844,13 @@ void emd_launch_stage(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
 
 void emd_launch_project(const OrbLayout &o, const TableSet &t, int n_atoms,
                         const void *u, double h3, double h_kb, double2 *c,
-                        void *hc, cudaStream_t st) {
+                        void *hc, cudaStream_t st, bool u_split) {
   if (n_atoms <= 0) return;
   emd_note_launches(1);
   if (o.prec == EMD_FP64) {
-    EMD_DISPATCH_BO(double, project_t, o, t, n_atoms, u, h3, h_kb, c, hc, st)
+    EMD_DISPATCH_BO(double, project_t, o, t, n_atoms, u, h3, h_kb, c, hc, st, u_split)
   } else {
-    EMD_DISPATCH_BO(float, project_t, o, t, n_atoms, u, h3, h_kb, c, hc, st)
+    EMD_DISPATCH_BO(float, project_t, o, t, n_atoms, u, h3, h_kb, c, hc, st, u_split)
   }
 }
 

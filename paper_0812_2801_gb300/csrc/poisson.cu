@@ -452,7 +452,7 @@ __global__ void k_lda(int n3, const double *rho, const double *vh,
 __global__ void k_veff(int n, double h, double L, const double *vloc,
                        const double *h0, const double *h1, const double *h2,
                        int hist_len, double field, double *ve, float *vef,
-                       float4 *vdiag, double w0) {
+                       float4 *vdiag, double w0, float2 *vsplit, double dvs, double dv0) {
   const int n3 = n * n * n;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n3) return;
@@ -470,6 +470,7 @@ __global__ void k_veff(int n, double h, double L, const double *vloc,
   }
   ve[i] = v;
   if (vef) vef[i] = (float)v;
+  if (vsplit) vsplit[i] = df_split(__fma_rn(dvs, v, dv0));
   if (vdiag) {
     const float d = (float)(w0 + v);
     vdiag[i] = make_float4(d, d, d, d);
@@ -642,11 +643,13 @@ void emd_launch_lda(int n3, const double *rho, const double *v_h,
 void emd_launch_veff(const GridInfo &g, const double *v_loc,
                      const double *const *hist, int hist_len, double field,
                      double *v_eff, float *v_eff_f, cudaStream_t st,
-                     float4 *v_diag, double w0) {
+                     float4 *v_diag, double w0, float2 *v_split, double dv_scale,
+                     double dv_shift) {
   emd_note_launches(1);
   k_veff<<<(g.n3 + 255) / 256, 256, 0, st>>>(
       g.n, g.h, g.L, v_loc, hist[0], hist_len > 1 ? hist[1] : hist[0],
-      hist_len > 2 ? hist[2] : hist[0], hist_len, field, v_eff, v_eff_f, v_diag, w0);
+      hist_len > 2 ? hist[2] : hist[0], hist_len, field, v_eff, v_eff_f, v_diag, w0,
+      v_split, dv_scale, dv_shift);
 }
 
 void emd_launch_dot_partials(int n3, const double *a, const double *b,
