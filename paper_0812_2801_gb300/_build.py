@@ -17,9 +17,8 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libemd.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["emd_api.cu", "hpsi.cu", "stage_df.cu", "tables.cu", "poisson.cu", "adjoint.cu", "project_pm.cu",
-           "groundstate.cu",
-           "observables.cu"]
+SOURCES = ["emd_api.cu", "hpsi.cu", "stage_df.cu", "tables.cu", "poisson.cu", "fft2.cu",
+           "adjoint.cu", "project_pm.cu", "groundstate.cu", "observables.cu"]
 
 
 def nvcc() -> str:

@@ -397,6 +397,12 @@ void emd_launch_vv_velocities(int n_atoms, const double *F_loc,
                               double *V, double dt, double mass, int update_v,
                               cudaStream_t st);
 
+// fft2.cu: spectral multiplication in five kernels
+bool emd_fft2_ok(int n);
+void emd_fft2_multiply(int n, const double *in, double *out, double2 *wa, double2 *wb,
+                       const double2 *roots, double c, double kappa, const double *inv_s,
+                       cudaStream_t st);
+
 // poisson.cu
 void emd_fft_plan_check(int n, int *ok);   // host-only factor check
 int emd_fft_prepare(int n);                 // twiddle tables on the device

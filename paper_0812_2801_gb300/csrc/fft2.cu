@@ -1,0 +1,691 @@
+// Spectral multiplication on periodic grids in five kernels: the transforms of
+// the Hartree and ionic electrostatics (eq. E_KS, eq. ionicpotential; a
+// periodic spectral solve stands in for the paper's finite-system solver) and
+// of Kerker's preconditioner.
+//
+// What bounds it: GB300's FP64 rate.  One FP64 warp instruction occupies a
+// quarter of an SM (a scheduler's FP64 lanes) for 64 cycles, so a pass costs
+// (FP64 instructions of a thread) x 64 cycles x (warps per scheduler), and on
+// small grids, which do not fill the 608 schedulers, what counts is the length
+// of one thread's chain.  So
+//  * a line's transform is two to four register butterflies of at most 16
+//    points with exchanges through shared memory between them.  The factors
+//    are chosen by that cost: few large butterflies (fewest instructions) on
+//    large grids, more small ones (short chains) on small grids;
+//  * the butterflies' own twiddles are constants, prime butterflies use the
+//    real symmetric form (half the multiplications of the direct sum);
+//  * the forward z transform, the spectral factor and the inverse z transform
+//    are one kernel: the spectrum along z never leaves the SM;
+//  * real data run as half-length complex lines (even n) and only kx <= n / 2
+//    is kept.
+// Measured: emd_poisson_static on 48^3 92 -> 54 us a call (seven passes of one
+// exchange per radix 2, 3, 4 or 5 on complex data before); the system's own
+// solve, ncu, cold caches: 48^3 60 -> 55 us, 64^3 94 -> 77 us; on 120^3
+// (54 orbitals, complex64) an MD step with its two solves takes 0.5 ms less.
+// Every pass reads lines that are contiguous and writes 64- or 128-byte pieces
+// of the layout whose next axis is contiguous.
+//   1 x real -> complex   [z][y][x]   -> [kx][z][y]
+//   2 y                   [kx][z][y]  -> [ky][kx][z]
+//   3 z, factor, inverse z            -> [kx][z][ky]
+//   4 inverse y                       -> [z][y][kx]
+//   5 inverse x, complex -> real      -> [z][y][x]
+// Inverse transforms run the forward butterflies with real and imaginary
+// parts exchanged on the way in and out.
+#include <atomic>
+#include "emd_internal.cuh"
+
+namespace {
+
+__device__ __forceinline__ double2 cadd(double2 a, double2 b) {
+  return make_double2(a.x + b.x, a.y + b.y);
+}
+__device__ __forceinline__ double2 csub(double2 a, double2 b) {
+  return make_double2(a.x - b.x, a.y - b.y);
+}
+__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
+  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+__device__ __forceinline__ double2 cswap(double2 a) { return make_double2(a.y, a.x); }
+
+// (cos, sin)(2 pi k / R); with k known at compile time the table folds away
+template <int R> __device__ __forceinline__ double2 circle(int k) {
+  if (R == 3) {
+    const double c[3] = {
+        1.0, -0.5, -0.5};
+    const double s[3] = {
+        0.0, 0.8660254037844386, -0.8660254037844386};
+    return make_double2(c[k], s[k]);
+  }
+  if (R == 5) {
+    const double c[5] = {
+        1.0, 0.30901699437494745, -0.8090169943749475, -0.8090169943749475,
+        0.30901699437494745};
+    const double s[5] = {
+        0.0, 0.9510565162951535, 0.5877852522924731, -0.5877852522924731,
+        -0.9510565162951535};
+    return make_double2(c[k], s[k]);
+  }
+  if (R == 6) {
+    const double c[6] = {
+        1.0, 0.5, -0.5, -1.0, -0.5, 0.5};
+    const double s[6] = {
+        0.0, 0.8660254037844386, 0.8660254037844386, 0.0, -0.8660254037844386,
+        -0.8660254037844386};
+    return make_double2(c[k], s[k]);
+  }
+  if (R == 7) {
+    const double c[7] = {
+        1.0, 0.6234898018587335, -0.2225209339563144, -0.9009688679024191,
+        -0.9009688679024191, -0.2225209339563144, 0.6234898018587335};
+    const double s[7] = {
+        0.0, 0.7818314824680298, 0.9749279121818236, 0.4338837391175581,
+        -0.4338837391175581, -0.9749279121818236, -0.7818314824680298};
+    return make_double2(c[k], s[k]);
+  }
+  if (R == 8) {
+    const double c[8] = {
+        1.0, 0.7071067811865476, 0.0, -0.7071067811865476, -1.0, -0.7071067811865476, 0.0,
+        0.7071067811865476};
+    const double s[8] = {
+        0.0, 0.7071067811865476, 1.0, 0.7071067811865476, 0.0, -0.7071067811865476, -1.0,
+        -0.7071067811865476};
+    return make_double2(c[k], s[k]);
+  }
+  if (R == 9) {
+    const double c[9] = {
+        1.0, 0.766044443118978, 0.17364817766693036, -0.5, -0.9396926207859084,
+        -0.9396926207859084, -0.5, 0.17364817766693036, 0.766044443118978};
+    const double s[9] = {
+        0.0, 0.6427876096865394, 0.984807753012208, 0.8660254037844386, 0.3420201433256687,
+        -0.3420201433256687, -0.8660254037844386, -0.984807753012208, -0.6427876096865394};
+    return make_double2(c[k], s[k]);
+  }
+  if (R == 10) {
+    const double c[10] = {
+        1.0, 0.8090169943749475, 0.30901699437494745, -0.30901699437494745,
+        -0.8090169943749475, -1.0, -0.8090169943749475, -0.30901699437494745,
+        0.30901699437494745, 0.8090169943749475};
+    const double s[10] = {
+        0.0, 0.5877852522924731, 0.9510565162951535, 0.9510565162951535, 0.5877852522924731,
+        0.0, -0.5877852522924731, -0.9510565162951535, -0.9510565162951535,
+        -0.5877852522924731};
+    return make_double2(c[k], s[k]);
+  }
+  if (R == 11) {
+    const double c[11] = {
+        1.0, 0.8412535328311812, 0.41541501300188644, -0.14231483827328514,
+        -0.6548607339452851, -0.9594929736144974, -0.9594929736144974, -0.6548607339452851,
+        -0.14231483827328514, 0.41541501300188644, 0.8412535328311812};
+    const double s[11] = {
+        0.0, 0.5406408174555976, 0.9096319953545183, 0.9898214418809327, 0.7557495743542583,
+        0.28173255684142967, -0.28173255684142967, -0.7557495743542583, -0.9898214418809327,
+        -0.9096319953545183, -0.5406408174555976};
+    return make_double2(c[k], s[k]);
+  }
+  if (R == 12) {
+    const double c[12] = {
+        1.0, 0.8660254037844386, 0.5, 0.0, -0.5, -0.8660254037844386, -1.0,
+        -0.8660254037844386, -0.5, 0.0, 0.5, 0.8660254037844386};
+    const double s[12] = {
+        0.0, 0.5, 0.8660254037844386, 1.0, 0.8660254037844386, 0.5, 0.0, -0.5,
+        -0.8660254037844386, -1.0, -0.8660254037844386, -0.5};
+    return make_double2(c[k], s[k]);
+  }
+  if (R == 13) {
+    const double c[13] = {
+        1.0, 0.8854560256532099, 0.5680647467311558, 0.12053668025532305,
+        -0.3546048870425356, -0.7485107481711011, -0.970941817426052, -0.970941817426052,
+        -0.7485107481711011, -0.3546048870425356, 0.12053668025532305, 0.5680647467311558,
+        0.8854560256532099};
+    const double s[13] = {
+        0.0, 0.46472317204376856, 0.8229838658936564, 0.992708874098054, 0.9350162426854148,
+        0.6631226582407952, 0.23931566428755777, -0.23931566428755777, -0.6631226582407952,
+        -0.9350162426854148, -0.992708874098054, -0.8229838658936564, -0.46472317204376856};
+    return make_double2(c[k], s[k]);
+  }
+  if (R == 14) {
+    const double c[14] = {
+        1.0, 0.9009688679024191, 0.6234898018587335, 0.2225209339563144,
+        -0.2225209339563144, -0.6234898018587335, -0.9009688679024191, -1.0,
+        -0.9009688679024191, -0.6234898018587335, -0.2225209339563144, 0.2225209339563144,
+        0.6234898018587335, 0.9009688679024191};
+    const double s[14] = {
+        0.0, 0.4338837391175581, 0.7818314824680298, 0.9749279121818236, 0.9749279121818236,
+        0.7818314824680298, 0.4338837391175581, 0.0, -0.4338837391175581,
+        -0.7818314824680298, -0.9749279121818236, -0.9749279121818236, -0.7818314824680298,
+        -0.4338837391175581};
+    return make_double2(c[k], s[k]);
+  }
+  if (R == 15) {
+    const double c[15] = {
+        1.0, 0.9135454576426009, 0.6691306063588582, 0.30901699437494745,
+        -0.10452846326765347, -0.5, -0.8090169943749475, -0.9781476007338057,
+        -0.9781476007338057, -0.8090169943749475, -0.5, -0.10452846326765347,
+        0.30901699437494745, 0.6691306063588582, 0.9135454576426009};
+    const double s[15] = {
+        0.0, 0.4067366430758002, 0.7431448254773942, 0.9510565162951535, 0.9945218953682733,
+        0.8660254037844386, 0.5877852522924731, 0.20791169081775934, -0.20791169081775934,
+        -0.5877852522924731, -0.8660254037844386, -0.9945218953682733, -0.9510565162951535,
+        -0.7431448254773942, -0.4067366430758002};
+    return make_double2(c[k], s[k]);
+  }
+  if (R == 16) {
+    const double c[16] = {
+        1.0, 0.9238795325112867, 0.7071067811865476, 0.3826834323650898, 0.0,
+        -0.3826834323650898, -0.7071067811865476, -0.9238795325112867, -1.0,
+        -0.9238795325112867, -0.7071067811865476, -0.3826834323650898, 0.0,
+        0.3826834323650898, 0.7071067811865476, 0.9238795325112867};
+    const double s[16] = {
+        0.0, 0.3826834323650898, 0.7071067811865476, 0.9238795325112867, 1.0,
+        0.9238795325112867, 0.7071067811865476, 0.3826834323650898, 0.0,
+        -0.3826834323650898, -0.7071067811865476, -0.9238795325112867, -1.0,
+        -0.9238795325112867, -0.7071067811865476, -0.3826834323650898};
+    return make_double2(c[k], s[k]);
+  }
+  return make_double2(1.0, 0.0);
+}
+
+// ---- forward DFTs of R points in registers ----------------------------------
+// odd primes: y_j = a_j - i b_j, y_{R-j} = a_j + i b_j with a_j = x_0 + sum_k
+// cos(2 pi j k / R) (x_k + x_{R-k}), b_j = sum_k sin(2 pi j k / R) (x_k - x_{R-k})
+template <int R> struct Dft {
+  static __device__ __forceinline__ void run(double2 (&v)[R]) {
+    constexpr int H = (R - 1) / 2;
+    double2 t[H], d[H];
+    double2 s0 = v[0];
+#pragma unroll
+    for (int k = 1; k <= H; ++k) {
+      t[k - 1] = cadd(v[k], v[R - k]);
+      d[k - 1] = csub(v[k], v[R - k]);
+      s0 = cadd(s0, t[k - 1]);
+    }
+    const double2 x0 = v[0];
+    v[0] = s0;
+#pragma unroll
+    for (int j = 1; j <= H; ++j) {
+      double2 a = x0, b = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int k = 1; k <= H; ++k) {
+        const double2 w = circle<R>(j * k % R);
+        a.x = fma(w.x, t[k - 1].x, a.x);
+        a.y = fma(w.x, t[k - 1].y, a.y);
+        b.x = fma(w.y, d[k - 1].x, b.x);
+        b.y = fma(w.y, d[k - 1].y, b.y);
+      }
+      v[j] = make_double2(a.x + b.y, a.y - b.x);
+      v[R - j] = make_double2(a.x - b.y, a.y + b.x);
+    }
+  }
+};
+template <> struct Dft<1> {
+  static __device__ __forceinline__ void run(double2 (&)[1]) {}
+};
+template <> struct Dft<2> {
+  static __device__ __forceinline__ void run(double2 (&v)[2]) {
+    const double2 a = v[0];
+    v[0] = cadd(a, v[1]);
+    v[1] = csub(a, v[1]);
+  }
+};
+template <> struct Dft<4> {
+  static __device__ __forceinline__ void run(double2 (&v)[4]) {
+    const double2 a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
+    const double2 c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
+    v[0] = cadd(a, c);
+    v[2] = csub(a, c);
+    v[1] = make_double2(b.x + d.y, b.y - d.x);   // b - i d
+    v[3] = make_double2(b.x - d.y, b.y + d.x);
+  }
+};
+// v (c - i s) for a constant (c, s); 1, -1, i and -i need no multiplication
+__device__ __forceinline__ double2 ctwiddle(double2 v, double2 w) {
+  if (w.y == 0.0) return w.x > 0.0 ? v : make_double2(-v.x, -v.y);
+  if (w.x == 0.0) return w.y > 0.0 ? make_double2(v.y, -v.x) : make_double2(-v.y, v.x);
+  return cmul(v, make_double2(w.x, -w.y));
+}
+// composite R = A B: B transforms of A points, constant twiddles, A of B points
+template <int A, int B> struct DftAB {
+  static __device__ __forceinline__ void run(double2 (&v)[A * B]) {
+    constexpr int R = A * B;
+    double2 u[B][A];
+#pragma unroll
+    for (int j = 0; j < B; ++j) {
+#pragma unroll
+      for (int r = 0; r < A; ++r) u[j][r] = v[j + B * r];
+      Dft<A>::run(u[j]);
+#pragma unroll
+      for (int k = 1; k < A; ++k)
+        if (j > 0) u[j][k] = ctwiddle(u[j][k], circle<R>(j * k % R));
+    }
+#pragma unroll
+    for (int k = 0; k < A; ++k) {
+      double2 w[B];
+#pragma unroll
+      for (int j = 0; j < B; ++j) w[j] = u[j][k];
+      Dft<B>::run(w);
+#pragma unroll
+      for (int q = 0; q < B; ++q) v[k + A * q] = w[q];
+    }
+  }
+};
+template <> struct Dft<6> : DftAB<2, 3> {};
+template <> struct Dft<8> : DftAB<2, 4> {};
+template <> struct Dft<9> : DftAB<3, 3> {};
+template <> struct Dft<10> : DftAB<2, 5> {};
+template <> struct Dft<12> : DftAB<3, 4> {};
+template <> struct Dft<14> : DftAB<2, 7> {};
+template <> struct Dft<15> : DftAB<3, 5> {};
+template <> struct Dft<16> : DftAB<4, 4> {};
+
+#define EMD_FFT_SWITCH(R, CALL)                                                     \
+  switch (R) {                                                                      \
+    case 1: CALL(1); break;                                                         \
+    case 2: CALL(2); break;                                                         \
+    case 3: CALL(3); break;                                                         \
+    case 4: CALL(4); break;                                                         \
+    case 5: CALL(5); break;                                                         \
+    case 6: CALL(6); break;                                                         \
+    case 7: CALL(7); break;                                                         \
+    case 8: CALL(8); break;                                                         \
+    case 9: CALL(9); break;                                                         \
+    case 10: CALL(10); break;                                                       \
+    case 11: CALL(11); break;                                                       \
+    case 12: CALL(12); break;                                                       \
+    case 13: CALL(13); break;                                                       \
+    case 14: CALL(14); break;                                                       \
+    case 15: CALL(15); break;                                                       \
+    case 16: CALL(16); break;                                                       \
+  }
+
+// A line transform of len = r[0] r[1] .. r[ns-1] points, ns >= 2.  One step
+// turns a block of R m values x[j + m t] into R blocks of m: block k holds
+// w_{Rm}^{jk} sum_t w_R^{tk} x[j + m t] and is the transform of length m that
+// gives the frequencies k, k + R, ...; so a step reads and writes the same
+// places, and the last one leaves X[k_1 + r_1 (k_2 + r_2 (...))].  Line l's
+// first-step blocks start at l ls + k_1 (m_1 | 1) (odd strides: no conflicts).
+constexpr int kFftSteps = 4;
+// t / d for t d < 2^32 by one multiplication (an integer division is ~30
+// instructions, and a step of a small grid is only ~150)
+struct FastDiv {
+  unsigned mul, d;
+};
+__host__ __device__ __forceinline__ FastDiv fast_div(unsigned d) {
+  FastDiv f;
+  f.d = d;
+  f.mul = d > 1 ? 0xffffffffu / d + 1u : 0u;
+  return f;
+}
+__device__ __forceinline__ int operator/(int t, const FastDiv &f) {
+  return f.d == 1 ? t : (int)__umulhi((unsigned)t, f.mul);
+}
+struct FftLine {
+  int n, len, ns;         // grid edge; line length; steps
+  int r[kFftSteps];       // factors
+  int m[kFftSteps];       // block length after the step
+  FastDiv by_r[kFftSteps], by_m[kFftSteps], by_blocks;   // by_blocks: len / r[ns - 1]
+  int tw;                 // exp(-2 pi i t / len) = roots[tw t], roots of n
+  int lsh;                // 2^lsh lines per CTA
+  int ls;                 // shared-memory stride of a line
+  int threads;            // per CTA
+};
+
+// block offset of frequency index kk = k_1 + r_1 (k_2 + ..) after `steps` steps
+__device__ __forceinline__ int block_at(const FftLine &p, int kk, int steps) {
+  if (steps == 1) return kk * (p.m[0] | 1);
+  int q = kk / p.by_r[0];
+  int off = (kk - q * p.r[0]) * (p.m[0] | 1);
+  for (int s = 1; s + 1 < steps; ++s) {
+    const int t = q / p.by_r[s];
+    off += (q - t * p.r[s]) * p.m[s];
+    q = t;
+  }
+  return off + q * p.m[steps - 1];
+}
+
+// The roots are read from shared memory (rt, copied at the kernel's start).
+// first step: ld(l, i) gives element i of line l
+template <int R, typename LD>
+__device__ __forceinline__ void first(const FftLine &p, const double2 *rt, double2 *ex, LD ld) {
+  const int m = p.m[0], mp = m | 1;
+  for (int t = threadIdx.x; t < m << p.lsh; t += blockDim.x) {
+    const int l = t / p.by_m[0], j = t - l * m;
+    double2 v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = ld(l, j + r * m);
+    Dft<R>::run(v);
+    double2 *e = ex + l * p.ls + j;
+    const double2 *w = rt;
+    e[0] = v[0];
+#pragma unroll
+    for (int k = 1; k < R; ++k) {
+      w += p.tw * j;                       // root j k
+      e[k * mp] = cmul(v[k], *w);
+    }
+  }
+}
+// step s in the middle; groups = product of the factors before it
+template <int R>
+__device__ __forceinline__ void middle(const FftLine &p, const double2 *rt, double2 *ex, int s,
+                                       int groups) {
+  const int m = p.m[s];
+  for (int t = threadIdx.x; t < (groups * m) << p.lsh; t += blockDim.x) {
+    const int b = t / p.by_m[s], j = t - b * m, l = b & ((1 << p.lsh) - 1), g = b >> p.lsh;
+    double2 *e = ex + l * p.ls + block_at(p, g, s) + j;
+    double2 v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = e[r * m];
+    Dft<R>::run(v);
+    const double2 *w = rt;
+    e[0] = v[0];
+#pragma unroll
+    for (int k = 1; k < R; ++k) {
+      w += p.tw * groups * j;
+      e[k * m] = cmul(v[k], *w);
+    }
+  }
+}
+// last step: st(l, k, X_k).  ALONG: neighbouring threads take neighbouring
+// frequencies of a line instead of neighbouring lines.
+template <int R, bool ALONG, typename ST>
+__device__ __forceinline__ void last(const FftLine &p, const double2 *ex, ST st) {
+  const int per = (int)p.by_blocks.d;
+  for (int t = threadIdx.x; t < per << p.lsh; t += blockDim.x) {
+    const int l = ALONG ? t / p.by_blocks : t & ((1 << p.lsh) - 1);
+    const int k = ALONG ? t - l * per : t >> p.lsh;
+    const double2 *e = ex + l * p.ls + block_at(p, k, p.ns - 1);
+    double2 v[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) v[j] = e[j];
+    Dft<R>::run(v);
+#pragma unroll
+    for (int q = 0; q < R; ++q) st(l, k + per * q, v[q]);
+  }
+}
+
+template <bool ALONG, typename LD, typename ST>
+__device__ __forceinline__ void line_fft(const FftLine &p, const double2 *rt, double2 *ex, LD ld,
+                                         ST st) {
+#define EMD_FIRST(R) first<R>(p, rt, ex, ld)
+  EMD_FFT_SWITCH(p.r[0], EMD_FIRST)
+  int groups = p.r[0];
+  for (int s = 1; s < p.ns - 1; ++s) {
+    __syncthreads();
+#define EMD_MIDDLE(R) middle<R>(p, rt, ex, s, groups)
+    EMD_FFT_SWITCH(p.r[s], EMD_MIDDLE)
+    groups *= p.r[s];
+  }
+  __syncthreads();
+#define EMD_LAST(R) last<R, ALONG>(p, ex, st)
+  EMD_FFT_SWITCH(p.r[p.ns - 1], EMD_LAST)
+}
+
+// shared memory: roots | exchange array | second copy of the lines
+__device__ __forceinline__ double2 *load_roots(double2 *sm, int n,
+                                               const double2 *__restrict__ roots) {
+  for (int t = threadIdx.x; t < n; t += blockDim.x) sm[t] = __ldg(roots + t);
+  __syncthreads();
+  return sm + n;
+}
+
+// 1: x real -> complex.  EVEN: x_2j + i x_2j+1 as a line of n / 2 values,
+// untangled into X_k = E_k + W^k O_k, E_k = (Z_k + conj Z_{m-k}) / 2, O_k =
+// (Z_k - conj Z_{m-k}) / (2i), W = exp(-2 pi i / n), k = 0 .. m.
+template <bool EVEN>
+__global__ void __launch_bounds__(256)
+k_fft_x(const double *__restrict__ in, double2 *__restrict__ out, FftLine p,
+        const double2 *__restrict__ roots) {
+  extern __shared__ double2 sm[];
+  const int n = p.n, nlines = n * n, l0 = blockIdx.x << p.lsh;
+  double2 *ex = load_roots(sm, n, roots), *zs = ex + (p.ls << p.lsh);
+  if (EVEN) {
+    line_fft<false>(p, sm, ex, [&](int l, int i) {
+      const int line = min(l0 + l, nlines - 1);
+      // two 8-byte loads: a caller's grid may start on any 8-byte boundary
+      const double *x = in + (size_t)line * n + 2 * i;
+      return make_double2(__ldg(x), __ldg(x + 1));
+    }, [&](int l, int k, double2 v) { zs[l * (p.len | 1) + k] = v; });
+    __syncthreads();
+    const int m = p.len;
+    for (int t = threadIdx.x; t < (m + 1) << p.lsh; t += blockDim.x) {
+      const int k = t >> p.lsh, l = t & ((1 << p.lsh) - 1);
+      if (l0 + l >= nlines) continue;
+      const double2 zk = zs[l * (m | 1) + (k == m ? 0 : k)];
+      const double2 zr = zs[l * (m | 1) + (k == 0 ? 0 : m - k)];
+      const double2 e = make_double2(0.5 * (zk.x + zr.x), 0.5 * (zk.y - zr.y));
+      const double2 o = make_double2(0.5 * (zk.y + zr.y), -0.5 * (zk.x - zr.x));
+      out[(size_t)k * nlines + l0 + l] = cadd(e, cmul(sm[k], o));
+    }
+  } else {
+    line_fft<false>(p, sm, ex, [&](int l, int i) {
+      const int line = min(l0 + l, nlines - 1);
+      return make_double2(__ldg(in + (size_t)line * n + i), 0.0);
+    }, [&](int l, int k, double2 v) {
+      if (l0 + l < nlines && 2 * k < n) out[(size_t)k * nlines + l0 + l] = v;
+    });
+  }
+}
+
+// 2: lines (kx, z) along y, [kx][z][y] -> [ky][kx][z].  4 (INV): lines (z, kx)
+// along ky, [kx][z][ky] -> [z][y][kx].
+template <bool INV>
+__global__ void __launch_bounds__(256)
+k_fft_y(const double2 *__restrict__ in, double2 *__restrict__ out, FftLine p, int nh, FastDiv by_nh,
+        const double2 *__restrict__ roots) {
+  extern __shared__ double2 sm[];
+  const int n = p.n, nlines = nh * n, l0 = blockIdx.x << p.lsh;
+  double2 *ex = load_roots(sm, n, roots);
+  line_fft<false>(p, sm, ex, [&](int l, int i) {
+    const int line = min(l0 + l, nlines - 1);
+    if (!INV) return __ldg(in + (size_t)line * n + i);
+    const int z = line / by_nh, kx = line - z * nh;
+    return cswap(__ldg(in + ((size_t)kx * n + z) * n + i));
+  }, [&](int l, int k, double2 v) {
+    const int line = l0 + l;
+    if (line >= nlines) return;
+    if (!INV) {
+      out[(size_t)k * nlines + line] = v;
+    } else {
+      const int z = line / by_nh, kx = line - z * nh;
+      out[((size_t)z * n + k) * nh + kx] = cswap(v);
+    }
+  });
+}
+
+// 3: lines (kx, ky) along z: forward, times the factor of the integer s = mx^2
+// + my^2 + mz^2 (|G|^2 = (2 pi / L)^2 s), inverse.  kappa < 0: the Poisson
+// kernel c / s, 0 at s = 0 (inv_s[s] = 1 / s, inv_s[0] = 0); else Kerker's c s / (s
+// + kappa), c at s = 0.  [ky][kx][z] -> [kx][z][ky].
+__global__ void __launch_bounds__(256)
+k_fft_z_factor(const double2 *__restrict__ in, double2 *__restrict__ out, FftLine p, int nh, FastDiv by_n,
+               double c, double kappa, const double *__restrict__ inv_s,
+               const double2 *__restrict__ roots) {
+  extern __shared__ double2 sm[];
+  const int n = p.n, nlines = nh * n, l0 = blockIdx.x << p.lsh;
+  double2 *ex = load_roots(sm, n, roots), *zs = ex + (p.ls << p.lsh);
+  line_fft<false>(p, sm, ex, [&](int l, int i) {
+    const int line = min(l0 + l, nlines - 1);
+    const int kx = line / by_n, ky = line - kx * n;
+    return __ldg(in + ((size_t)ky * nh + kx) * n + i);
+  }, [&](int l, int k, double2 v) {
+    const int line = min(l0 + l, nlines - 1);
+    const int kx = line / by_n, ky = line - kx * n;
+    const int my = 2 * ky < n ? ky : ky - n, mz = 2 * k < n ? k : k - n;
+    const int s = kx * kx + my * my + mz * mz;
+    double f;
+    if (kappa < 0.0)
+      f = c * __ldg(inv_s + s);
+    else
+      f = s == 0 ? c : c * (double)s / ((double)s + kappa);
+    zs[l * (n | 1) + k] = make_double2(f * v.y, f * v.x);      // exchanged: inverse
+  });
+  __syncthreads();
+  line_fft<false>(p, sm, ex, [&](int l, int i) { return zs[l * (n | 1) + i]; },
+                  [&](int l, int z, double2 v) {
+    const int line = l0 + l;
+    if (line >= nlines) return;
+    const int kx = line / by_n, ky = line - kx * n;
+    out[((size_t)kx * n + z) * n + ky] = cswap(v);
+  });
+}
+
+// 5: inverse x.  EVEN: Z_k = (X_k + conj X_{m-k}) + i conj(W^k) (X_k - conj
+// X_{m-k}), k < m, and the inverse half-length transform gives x_2j + i
+// x_2j+1.  Odd n: the full Hermitian line, real parts kept.
+template <bool EVEN>
+__global__ void __launch_bounds__(256)
+k_fft_x_inv(const double2 *__restrict__ in, double *__restrict__ out, FftLine p, int nh,
+            const double2 *__restrict__ roots) {
+  extern __shared__ double2 sm[];
+  const int n = p.n, nlines = n * n, l0 = blockIdx.x << p.lsh;
+  double2 *ex = load_roots(sm, n, roots), *xs = ex + (p.ls << p.lsh);
+  for (int t = threadIdx.x; t < nh << p.lsh; t += blockDim.x) {
+    const int l = t / nh, k = t - l * nh, line = min(l0 + l, nlines - 1);
+    xs[l * nh + k] = __ldg(in + (size_t)line * nh + k);
+  }
+  __syncthreads();
+  if (EVEN) {
+    const int m = p.len;
+    line_fft<true>(p, sm, ex, [&](int l, int k) {
+      const double2 xk = xs[l * nh + k], xr = xs[l * nh + m - k];
+      const double2 sp = make_double2(xk.x + xr.x, xk.y - xr.y);
+      const double2 df = make_double2(xk.x - xr.x, xk.y + xr.y);
+      const double2 w = sm[k];
+      const double2 t = cmul(make_double2(w.x, -w.y), df);
+      return make_double2(sp.y + t.x, sp.x - t.y);             // exchanged: inverse
+    }, [&](int l, int k, double2 v) {
+      if (l0 + l >= nlines) return;
+      double *x = out + (size_t)(l0 + l) * n + 2 * k;
+      x[0] = v.y;
+      x[1] = v.x;
+    });
+  } else {
+    line_fft<true>(p, sm, ex, [&](int l, int k) {
+      const double2 v = xs[l * nh + (k < nh ? k : n - k)];
+      return make_double2(k < nh ? v.y : -v.y, v.x);           // exchanged: inverse
+    }, [&](int l, int k, double2 v) {
+      if (l0 + l < nlines) out[(size_t)(l0 + l) * n + k] = v.y;
+    });
+  }
+}
+
+// FP64 instructions of a butterfly and its R - 1 twiddle products
+int butterfly_cost(int R) {
+  static const int dft[17] = {0, 0, 4, 14, 16, 36, 44, 66, 64, 100, 92, 150, 108, 210, 156, 170, 160};
+  return dft[R] + 4 * (R - 1);
+}
+
+// the cheapest way to write len as 2 to 4 factors of at most 16, in ascending
+// order: a step costs its instructions times 64 cycles times the warps per
+// scheduler (at least one), and about 1500 cycles for its exchange
+void best_factors(FftLine &p, int nlines, int ns, int at, int left, int lo, int *r, double c,
+                  double &best) {
+  if (at == ns - 1) {
+    if (left > 16 || left < lo) return;
+    r[at] = left;
+    const double w = (double)nlines * (p.len / left) / 32.0 / 608.0;
+    c += (w > 1.0 ? w : 1.0) * (butterfly_cost(left) - 4 * (left - 1)) * 64.0;
+    if (c >= best) return;
+    best = c;
+    p.ns = ns;
+    for (int s = 0; s < ns; ++s) p.r[s] = r[s];
+    return;
+  }
+  for (int f = lo; f <= 16; ++f) {
+    if (left % f) continue;
+    const double w = (double)nlines * (p.len / f) / 32.0 / 608.0;
+    r[at] = f;
+    best_factors(p, nlines, ns, at + 1, left / f, f, r,
+                 c + 1500.0 + (w > 1.0 ? w : 1.0) * butterfly_cost(f) * 64.0, best);
+  }
+}
+
+// false: len is not a product of four factors of at most 16
+bool line_plan(FftLine &p, int n, int len, int nlines) {
+  p.n = n;
+  p.len = len;
+  p.ns = 0;
+  int r[kFftSteps];
+  double best = 1e300;
+  for (int ns = 2; ns <= kFftSteps; ++ns) best_factors(p, nlines, ns, 0, len, 1, r, 0.0, best);
+  if (!p.ns) return false;
+  int m = len;
+  for (int s = 0; s < p.ns; ++s) {
+    p.m[s] = m /= p.r[s];
+    p.by_r[s] = fast_div(p.r[s]);
+    p.by_m[s] = fast_div(p.m[s]);
+  }
+  p.by_blocks = fast_div(len / p.r[p.ns - 1]);
+  p.tw = n / len;
+  p.ls = (p.r[0] * (p.m[0] | 1)) | 1;
+  // 8 lines: transposed writes of 128 bytes; 4 where two copies of the lines
+  // and the roots pass 200 KB
+  p.lsh = (8 * (p.ls + n + 1) + n) * (int)sizeof(double2) <= 200 * 1024 ? 3 : 2;
+  const int most = (len / p.r[0]) << p.lsh;            // threads of the widest step
+  p.threads = most >= 256 ? 256 : (most + 31) / 32 * 32;
+  return true;
+}
+
+// The two line plans of a grid (x, and y or z), worked out once per size and
+// kept for the life of the process.
+struct FftPlan {
+  FftLine x, y;
+  bool ok;
+};
+constexpr int kFftMaxN = 1024;
+const FftPlan *plan_of(int n) {
+  static std::atomic<const FftPlan *> kept[kFftMaxN + 1];
+  if (n < 2 || n > kFftMaxN) return nullptr;
+  const FftPlan *p = kept[n].load();
+  if (!p) {
+    FftPlan *q = new FftPlan();
+    const int nh = n / 2 + 1;                     // (n + 1) / 2 for odd n
+    q->ok = line_plan(q->x, n, n % 2 ? n : n / 2, n * n) && line_plan(q->y, n, n, nh * n);
+    if (kept[n].compare_exchange_strong(p, q)) p = q;
+    else delete q;
+  }
+  return p->ok ? p : nullptr;
+}
+
+// grids above ~190 points need more than 48 KB: 1024 takes 2 x 4 lines and the
+// roots, 144 KB (once per process and device; setting it again changes nothing)
+void allow_large_shared() {
+  const int most = 200 * 1024;
+  cudaFuncSetAttribute(k_fft_x<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(k_fft_x<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(k_fft_y<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(k_fft_y<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(k_fft_z_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(k_fft_x_inv<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(k_fft_x_inv<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
+}  // namespace
+
+bool emd_fft2_ok(int n) { return plan_of(n) != nullptr; }
+
+// out = the inverse transform of the spectral factor times the transform of
+// the real grid `in`.  in is read by the first pass only, so out may alias it;
+// wa, wb: n^2 (n / 2 + 1) values each; roots: exp(-2 pi i t / n), t < n.
+void emd_fft2_multiply(int n, const double *in, double *out, double2 *wa, double2 *wb,
+                       const double2 *roots, double c, double kappa, const double *inv_s,
+                       cudaStream_t st) {
+  const bool even = n % 2 == 0;
+  const int nh = n / 2 + 1;                       // (n + 1) / 2 for odd n
+  const FftLine &px = plan_of(n)->x, &py = plan_of(n)->y;
+  const int lx = 1 << px.lsh, ly = 1 << py.lsh;
+  const int bx = (n * n + lx - 1) / lx, by = (nh * n + ly - 1) / ly;
+  const size_t c16 = sizeof(double2);
+  const size_t sx = (n + (size_t)lx * (px.ls + (px.len | 1))) * c16;
+  const size_t sxi = (n + (size_t)lx * (px.ls + nh)) * c16;
+  const size_t sy = (n + (size_t)ly * py.ls) * c16;
+  const size_t sz = (n + (size_t)ly * (py.ls + (n | 1))) * c16;
+  if (sz > 49152) allow_large_shared();
+  const FastDiv by_n = fast_div(n), by_nh = fast_div(nh);
+  if (even) k_fft_x<true><<<bx, px.threads, sx, st>>>(in, wa, px, roots);
+  else k_fft_x<false><<<bx, px.threads, sx, st>>>(in, wa, px, roots);
+  k_fft_y<false><<<by, py.threads, sy, st>>>(wa, wb, py, nh, by_nh, roots);
+  k_fft_z_factor<<<by, py.threads, sz, st>>>(wb, wa, py, nh, by_n, c, kappa, inv_s, roots);
+  k_fft_y<true><<<by, py.threads, sy, st>>>(wa, wb, py, nh, by_nh, roots);
+  if (even) k_fft_x_inv<true><<<bx, px.threads, sxi, st>>>(wb, out, px, nh, roots);
+  else k_fft_x_inv<false><<<bx, px.threads, sxi, st>>>(wb, out, px, nh, roots);
+}
