@@ -683,7 +683,7 @@ int emd_init_system(const emd_config *cfg, emd_system **out) {
     TRY(A((void **)&t.tile_atoms, (size_t)ntiles * EMD_TILE_ATOM_MAX * 4));
     TRY(A((void **)&t.tile_off, ntiles * 4));
     TRY(A((void **)&t.at_ntiles, na * 4));
-    TRY(A((void **)&t.at_tiles, (size_t)na * ntiles * sizeof(int2)));
+    TRY(A((void **)&t.at_rows, (size_t)na * ntiles * 4));
     TRY(A((void **)&t.g_ion, n3 * 8));
     t.gtab = nullptr;
     t.glo = nullptr;
@@ -722,13 +722,11 @@ int emd_init_system(const emd_config *cfg, emd_system **out) {
   TRY(A((void **)&s->err, sizeof(int)));
   TRY(A((void **)&s->occ_w, (size_t)o.n_orb_pad * 8));
   TRY(A((void **)&s->occ_winv, (size_t)o.n_orb_pad * 8));
-  if (c.precision == EMD_FP64 && o.bo == 2) {
-    TRY(A((void **)&o.gs.part, (size_t)kGatherMaxCtas * 16 * 8));
-    TRY(A((void **)&o.gs.arrived, (size_t)kGatherMaxCtas / 2 * 4));
-    TRY(cudaMemset(o.gs.arrived, 0, (size_t)kGatherMaxCtas / 2 * 4) == cudaSuccess
-            ? EMD_OK
-            : fail(EMD_ECUDA, "cudaMemset failed"));
-  }
+  TRY(A((void **)&o.gs.part, (size_t)kGatherMaxCtas * 16 * 8));
+  TRY(A((void **)&o.gs.arrived, (size_t)kGatherMaxCtas / 2 * 4));
+  TRY(cudaMemset(o.gs.arrived, 0, (size_t)kGatherMaxCtas / 2 * 4) == cudaSuccess
+          ? EMD_OK
+          : fail(EMD_ECUDA, "cudaMemset failed"));
   s->f.assign(o.n_orb, c.occ);
 #undef TRY
   cudaError_t e = cudaMemsetAsync(s->err, 0, sizeof(int), s->st);

@@ -131,7 +131,8 @@ struct TableSet {
   int *tile_atoms;  // [n_tiles][EMD_TILE_ATOM_MAX] in atom order
   int *tile_off;    // [n_tiles] exclusive prefix sum of tile_nat
   int *at_ntiles;   // [n_atoms] tiles listing the atom
-  int2 *at_tiles;   // [n_atoms][n_tiles] (tile, slot) in tile order
+  int *at_rows;     // [n_atoms][n_tiles] rows tile_off + slot of the per-tile
+                    // partials that belong to the atom, in tile order
   int n_slots_cap;  // n_tiles * EMD_TILE_ATOM_MAX
   double *g_ion;    // [n3] sum of Gaussian ion charges
   // separable ion Gaussian: exp(-d_a^2 / a^2) per atom, image and axis along
@@ -496,7 +497,7 @@ struct OrbLayout {
   // the same stencil as integers over a common denominator: c_k = num_k / den
   // (the double-float FP64 stage accumulates with these, exact in FP32)
   double num[EMD_MAX_HALF_ORDER + 1], den;
-  GatherScratch gs;    // complex128, bo = 2
+  GatherScratch gs;
   // the double-float stage's diagonal dv = dv_shift + dv_scale v_eff
   double dv_scale() const { return -2.0 * h * h * den; }
   double dv_shift() const { return 3.0 * num[0]; }

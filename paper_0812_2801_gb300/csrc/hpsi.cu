@@ -1498,13 +1498,25 @@ k_nl_force_df(const double2 *__restrict__ u, size_t n3, int n_blk,
 
 // ---- dispatch -------------------------------------------------------------
 
-// planes per z-chunk of a marching stage launch: the caller's choice, else
-// whole columns unless the columns alone would leave SMs idle (each chunk
-// restages and re-stencils 2M halo planes)
-inline int stage_zchunk(const OrbLayout &o, int cols, int min_ctas) {
+// planes per z-chunk of a marching stage launch: the caller's choice, else the
+// split with the smallest estimated time.  A chunk restages and re-stencils 2M
+// halo planes and fills its ring (about two planes more); one CTA per SM, so
+// the chunks run in rounds of 152.  (At least 304 CTAs or 16 planes per chunk,
+// the earlier rule, gave 108 CTAs of 24 planes on 16 orbitals of 48^3: 33 us;
+// this gives 144 of 20.)
+inline int stage_zchunk(const OrbLayout &o, int cols) {
   if (o.zchunk > 0) return std::min(o.zchunk, o.n);
-  const int nz = std::max(1, std::min((min_ctas + cols - 1) / cols, o.n / 16));
-  return (o.n + nz - 1) / nz;
+  int best = o.n;
+  long cost = 0;
+  for (int nz = 1; nz <= std::max(1, o.n / 4); ++nz) {
+    const int zc = (o.n + nz - 1) / nz, ctas = cols * ((o.n + zc - 1) / zc);
+    const long c = (long)((ctas + 151) / 152) * (zc + 2 * o.half_order + 2);
+    if (nz == 1 || c < cost) {
+      cost = c;
+      best = zc;
+    }
+  }
+  return best;
 }
 
 template <typename T, int BO, int M>
@@ -1604,9 +1616,7 @@ void stage_c_tt(const OrbLayout &o, const StageArgs &a, size_t smem, cudaStream_
     attr_done = true;
   }
   const int ntx = (o.n + Z::TX - 1) / Z::TX, nty = (o.n + Z::TY - 1) / Z::TY;
-  // one z-chunk per column unless the columns alone would leave SMs idle:
-  // each chunk restages and re-stencils 2M halo planes
-  const int zc = stage_zchunk(o, ntx * nty * o.n_blk, 2 * 152);
+  const int zc = stage_zchunk(o, ntx * nty * o.n_blk);
   dim3 grid(ntx * nty, (o.n + zc - 1) / zc, o.n_blk);
   k_stage_c<BO, M, HCS, TMA><<<grid, Z::NT, smem + 256, st>>>(
       (const float2 *)a.u_in, (const float2 *)a.psi0, (float2 *)a.u_out,

@@ -58,8 +58,8 @@ __global__ void k_tile_offsets(const int *tile_nat, int ntiles, int *tile_off) {
 
 // For atom J: the (tile, slot) pairs of the tiles listing J, in tile order.
 __global__ void __launch_bounds__(256)
-k_atom_tiles(const int *tile_nat, const int *tile_atoms, int ntiles, int cap,
-             int *at_ntiles, int2 *at_tiles, int *err) {
+k_atom_tiles(const int *tile_nat, const int *tile_atoms, const int *tile_off, int ntiles, int cap,
+             int *at_ntiles, int *at_rows, int *err) {
   __shared__ int warp_tot[8];
   __shared__ int s_base;
   const int J = blockIdx.x;
@@ -83,7 +83,7 @@ k_atom_tiles(const int *tile_nat, const int *tile_atoms, int ntiles, int cap,
     }
     if (hit) {
       const int e = off + __popc(m & ((1u << lane) - 1u));
-      if (e < cap) at_tiles[(size_t)J * cap + e] = make_int2(t, slot);
+      if (e < cap) at_rows[(size_t)J * cap + e] = tile_off[t] + slot;
       else atomicOr(err, EMD_ERRBIT_AT);
     }
     __syncthreads();
@@ -180,8 +180,7 @@ k_project_pm(const typename cplx<T>::type *__restrict__ u, int n, int nt,
 template <typename T, int BO>
 __global__ void k_project_pm_reduce(const double2 *__restrict__ partial,
                                     const int *__restrict__ at_ntiles,
-                                    const int2 *__restrict__ at_tiles, int cap,
-                                    const int *__restrict__ tile_off,
+                                    const int *__restrict__ at_rows, int cap,
                                     int n_slots_total, int n_orb_pad, double h3,
                                     double h_kb, double2 *c,
                                     typename cplx<T>::type *hc) {
@@ -193,8 +192,7 @@ __global__ void k_project_pm_reduce(const double2 *__restrict__ partial,
   double re = 0.0, im = 0.0;
   const int m = at_ntiles[J];
   for (int i = 0; i < m; ++i) {
-    const int2 ts = at_tiles[(size_t)J * cap + i];
-    const double2 v = partial[((size_t)blk * n_slots_total + tile_off[ts.x] + ts.y) * BO + j];
+    const double2 v = partial[((size_t)blk * n_slots_total + at_rows[(size_t)J * cap + i]) * BO + j];
     re += v.x;
     im += v.y;
   }
@@ -217,8 +215,8 @@ void project_pm_t(const OrbLayout &o, const TableSet &t, int n_atoms, const void
                                            t.pt_p, t.tile_nat, t.tile_atoms,
                                            t.tile_off, t.n_slots_cap, partial);
   dim3 g2(n_atoms, (o.n_orb_pad + 127) / 128);
-  k_project_pm_reduce<T, BO><<<g2, 128, 0, st>>>(partial, t.at_ntiles, t.at_tiles,
-                                                nt * nt * nt, t.tile_off, t.n_slots_cap,
+  k_project_pm_reduce<T, BO><<<g2, 128, 0, st>>>(partial, t.at_ntiles, t.at_rows,
+                                                nt * nt * nt, t.n_slots_cap,
                                                 o.n_orb_pad, h3, h_kb, c, (V *)hc);
 }
 
@@ -362,38 +360,47 @@ k_tile_gather(const float2 *__restrict__ u, int n, int nt, int n_orb_pad,
   }
 }
 
-// c[J][A] = h^3 sum over J's (tile, slot) list; hc = h_kb c.  Block
-// (atom, 32 orbitals), 8 warps: warp w adds the list entries i = w mod 8 in
-// increasing order (lane = orbital), then the 8 warp sums are added in warp
-// order (deterministic).
+// c[J][A] = h^3 sum over J's rows of the partials; hc = h_kb c.  Block (atom,
+// OW orbitals): the 256 threads are 256 / OW slices of OW orbitals, slice k
+// adds the rows k, k + 256 / OW, ...; then the slices of a warp (fixed tree)
+// and the warps (in order) are added.  Narrow groups, because the length of a
+// slice's chain and the FP64 adds of one SM are the cost: 32 orbitals per
+// block left 8 blocks of 27 rows per warp on 8 atoms and 16 orbitals (13.2
+// us; 48^3 grid, 8 launches a step).
+template <int OW>
 __global__ void __launch_bounds__(256)
 k_project_tile_reduce(const double2 *__restrict__ partial, const int *__restrict__ at_ntiles,
-                      const int2 *__restrict__ at_tiles, int cap,
-                      const int *__restrict__ tile_off, int n_orb_pad, int n_orb_used,
+                      const int *__restrict__ at_rows, int cap, int n_orb_pad, int n_orb_used,
                       double h3, double h_kb, double2 *c, float2 *hc) {
-  __shared__ double2 ws[8][32];
+  constexpr int NSL = 256 / OW;
+  __shared__ double2 ws[8][OW];
   const int J = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int A = blockIdx.y * 32 + lane;
+  const int A = blockIdx.y * OW + threadIdx.x % OW;
   const int m = at_ntiles[J];
+  const int *rows = at_rows + (size_t)J * cap;
   double re = 0.0, im = 0.0;
   if (A < n_orb_used) {
 #pragma unroll 4
-    for (int i = warp; i < m; i += 8) {
-      const int2 ts = __ldg(at_tiles + (size_t)J * cap + i);
-      const double2 v = partial[((size_t)__ldg(tile_off + ts.x) + ts.y) * n_orb_pad + A];
+    for (int i = threadIdx.x / OW; i < m; i += NSL) {
+      const double2 v = partial[(size_t)__ldg(rows + i) * n_orb_pad + A];
       re += v.x;
       im += v.y;
     }
   }
-  ws[warp][lane] = make_double2(re, im);
+#pragma unroll
+  for (int o = 16; o >= OW; o >>= 1) {
+    re += __shfl_xor_sync(0xffffffffu, re, o);
+    im += __shfl_xor_sync(0xffffffffu, im, o);
+  }
+  if (lane < OW) ws[warp][lane] = make_double2(re, im);
   __syncthreads();
-  if (warp == 0 && A < n_orb_used) {
+  if (threadIdx.x < OW && A < n_orb_used) {
     re = 0.0;
     im = 0.0;
     for (int w = 0; w < 8; ++w) {
-      re += ws[w][lane].x;
-      im += ws[w][lane].y;
+      re += ws[w][threadIdx.x].x;
+      im += ws[w][threadIdx.x].y;
     }
     const size_t o = (size_t)J * n_orb_pad + A;
     c[o] = make_double2(h3 * re, h3 * im);
@@ -401,35 +408,34 @@ k_project_tile_reduce(const double2 *__restrict__ partial, const int *__restrict
   }
 }
 
-// F_J = coef sum_A Re(conj(c_JA) h^3 dc_JA), dc summed over J's tiles in
-// tile order; one block per atom, orbitals over threads, fixed-tree sum.
-__global__ void __launch_bounds__(128)
+// F_J = coef h^3 sum over J's rows and the orbitals of Re(conj(c_JA) dc_row,A):
+// the product is linear in dc, so every (row, orbital) pair goes straight into
+// three sums; `split` CTAs per atom share the pairs.  (One block per atom that
+// first added each orbital's rows took 89 us on 8 atoms and 16 orbitals: 216
+// rows in a chain, 16 of 128 threads at work.)
+__global__ void __launch_bounds__(256)
 k_nl_force_tile_reduce(const double2 *__restrict__ partial, const int *__restrict__ at_ntiles,
-                       const int2 *__restrict__ at_tiles, int cap,
-                       const int *__restrict__ tile_off, const double2 *__restrict__ c,
-                       int n_orb, int n_orb_pad, double h3, double coef, double *F) {
-  __shared__ double red[4 * 3];
-  const int J = blockIdx.x;
-  const int m = at_ntiles[J];
-  double f[3] = {0.0, 0.0, 0.0};
-  for (int A = threadIdx.x; A < n_orb; A += blockDim.x) {
-    double dr[3] = {0.0, 0.0, 0.0}, di[3] = {0.0, 0.0, 0.0};
-    for (int i = 0; i < m; ++i) {
-      const int2 ts = at_tiles[(size_t)J * cap + i];
-      const double2 *v = partial + (((size_t)tile_off[ts.x] + ts.y) * n_orb_pad + A) * 3;
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        dr[a] += v[a].x;
-        di[a] += v[a].y;
-      }
-    }
+                       const int *__restrict__ at_rows, int cap, const double2 *__restrict__ c,
+                       int n_orb, int n_orb_pad, double coef, int split, GatherScratch gs,
+                       double *F) {
+  __shared__ double red[8 * 4], res[4];
+  const int J = blockIdx.x, rank = blockIdx.y;
+  const int total = at_ntiles[J] * n_orb;
+  const int *rows = at_rows + (size_t)J * cap;
+  double f[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+  for (int q = rank * 256 + threadIdx.x; q < total; q += split * 256) {
+    const int i = q / n_orb, A = q - i * n_orb;
+    const double2 *v = partial + ((size_t)__ldg(rows + i) * n_orb_pad + A) * 3;
     const double2 cj = c[(size_t)J * n_orb_pad + A];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) f[a] += cj.x * (h3 * dr[a]) + cj.y * (h3 * di[a]);
+    for (int a = 0; a < 3; ++a) {
+      const double2 d = v[a];
+      f[a] = fma(cj.x, d.x, fma(cj.y, d.y, f[a]));
+    }
   }
-  emd_block_sum<3>(f, red);
-  if (threadIdx.x == 0)
-    for (int a = 0; a < 3; ++a) F[3 * J + a] = coef * f[a];
+  if (!emd_split_sum<4>(f, red, res, gs, J, rank, split)) return;
+  if (threadIdx.x < 3) F[3 * J + threadIdx.x] = coef * res[threadIdx.x];
 }
 
 template <int BO, bool FORCE>
@@ -453,8 +459,8 @@ void emd_launch_tile_atoms(const GridInfo &g, int n_atoms, TableSet &t, int *err
                                                      t.tile_nat, t.tile_atoms, err);
   k_tile_offsets<<<1, 1024, 0, st>>>(t.tile_nat, ntiles, t.tile_off);
   if (n_atoms > 0)
-    k_atom_tiles<<<n_atoms, 256, 0, st>>>(t.tile_nat, t.tile_atoms, ntiles, ntiles,
-                                          t.at_ntiles, t.at_tiles, err);
+    k_atom_tiles<<<n_atoms, 256, 0, st>>>(t.tile_nat, t.tile_atoms, t.tile_off, ntiles, ntiles,
+                                          t.at_ntiles, t.at_rows, err);
 }
 
 void emd_launch_project_pm(const OrbLayout &o, const TableSet &t, int n_atoms,
@@ -489,10 +495,15 @@ void emd_launch_project_tile(const OrbLayout &o, const TableSet &t, int n_atoms,
   }
   const int nt = (o.n + EMD_TILE - 1) / EMD_TILE;
   const int used = o.n_blk * o.bo;
-  dim3 g2(n_atoms, (used + 31) / 32);
-  k_project_tile_reduce<<<g2, 256, 0, st>>>(partial, t.at_ntiles, t.at_tiles, nt * nt * nt,
-                                           t.tile_off, o.n_orb_pad, used, h3, h_kb, c,
-                                           (float2 *)hc);
+  // 8 orbitals per block read 128-byte pieces; 4 where 8 leave SMs idle
+  if (n_atoms * ((used + 7) / 8) >= 2 * 152)
+    k_project_tile_reduce<8><<<dim3(n_atoms, (used + 7) / 8), 256, 0, st>>>(
+        partial, t.at_ntiles, t.at_rows, nt * nt * nt, o.n_orb_pad, used, h3, h_kb, c,
+        (float2 *)hc);
+  else
+    k_project_tile_reduce<4><<<dim3(n_atoms, (used + 3) / 4), 256, 0, st>>>(
+        partial, t.at_ntiles, t.at_rows, nt * nt * nt, o.n_orb_pad, used, h3, h_kb, c,
+        (float2 *)hc);
 }
 
 void emd_launch_nl_force_tile(const OrbLayout &o, const TableSet &t, int n_atoms,
@@ -506,7 +517,10 @@ void emd_launch_nl_force_tile(const OrbLayout &o, const TableSet &t, int n_atoms
     case 4: tile_gather_t<4, true>(o, t, u, partial, st); break;
   }
   const int nt = (o.n + EMD_TILE - 1) / EMD_TILE;
-  k_nl_force_tile_reduce<<<n_atoms, 128, 0, st>>>(partial, t.at_ntiles, t.at_tiles,
-                                                 nt * nt * nt, t.tile_off, c, o.n_orb,
-                                                 o.n_orb_pad, h3, coef, F_nl);
+  // an atom's rows: about (2 r / (8 h) + 1)^3 tiles; the split keeps at least
+  // four rounds of the loop per CTA
+  const int split = emd_gather_split(n_atoms, 2 * o.n_orb * 128);
+  k_nl_force_tile_reduce<<<dim3(n_atoms, split), 256, 0, st>>>(
+      partial, t.at_ntiles, t.at_rows, nt * nt * nt, c, o.n_orb, o.n_orb_pad, coef * h3, split,
+      o.gs, F_nl);
 }
