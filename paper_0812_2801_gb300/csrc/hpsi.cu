@@ -136,10 +136,17 @@ k_stage(const typename cplx<T>::type *__restrict__ u_in,
 // rows, so y-neighbours come from a register window (RY + 2M loads for RY
 // outputs) and x-neighbours from shared memory (2M loads per output).
 // ---------------------------------------------------------------------------
+//
+// The tile: 256 threads, 16 x 8 points at bo = 4, two CTAs per SM.  The kernel
+// is bound by shared-memory wavefronts (~48 SM cycles per 32 updates of the 65
+// it takes) and by waits for them; two half-size CTAs do not meet at one
+// barrier.  One CTA of 512 threads (16 x 16 points, 2.25 instead of 3 staged
+// values per update) took 0.862 ms per launch on 96^3 x 128 orbitals against
+// 0.815, and 0.797 against 0.768 ms on 120^3 x 54.
 template <int BO, int M> struct ZTile {
   static constexpr int NC = 64;                 // orbital columns = threads in x
   static constexpr int TX = NC / BO;            // points per tile in x
-  static constexpr int NT = 512;                // threads per CTA
+  static constexpr int NT = 256;                // threads per CTA
   static constexpr int TYT = NT / NC;           // thread rows
   static constexpr int RY = 2;                  // grid rows per thread
   static constexpr int TY = TYT * RY;           // grid rows per tile
@@ -460,7 +467,7 @@ template <int BO, int M> struct ZCTile : ZTile<BO, M> {
 // one thread and completing on the ring slot's mbarrier; the orbital plane
 // with its periodic halo keeps the per-thread cp.async chunks.
 template <int BO, int M, bool HCS, bool TMA>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(256, 2)
 k_stage_c(const float2 *__restrict__ u_in, const float2 *__restrict__ psi0,
           float2 *__restrict__ u_out, const float4 *__restrict__ diag,
           const int2 *__restrict__ pt4, const int *__restrict__ pt_J,
@@ -612,6 +619,8 @@ k_stage_c(const float2 *__restrict__ u_in, const float2 *__restrict__ psi0,
     oval[r] = x < n && y < n;
     orow[r] = (y * n + x) * BO + j;
   }
+  // warps with no point of the grid (tiles that overhang its edge) only stage
+  const bool active = __any_sync(0xffffffffu, oval[0]);
   const int win0 = ((tyr * RY) * Z::SW + xl + M) * BO + j;     // float2 index
   const int pnt0 = (tyr * RY) * Z::TX + xl;
 
@@ -638,6 +647,7 @@ k_stage_c(const float2 *__restrict__ u_in, const float2 *__restrict__ psi0,
       if (TMA && !mbar_wait_bounded(mb0 + 8 * sb, (unsigned)(zi / 3) & 1u)) timed_out = true;
       __syncthreads();
       if (zi + 2 < total) issue(zi + 2, (ph + 2) % 3);
+      if (!active) continue;
       const unsigned char *base = smraw + sb * Z::SLOT;
       const float2 *P = reinterpret_cast<const float2 *>(base);
       const float2 *DP = reinterpret_cast<const float2 *>(base + Z::UB);   // (d, d) at 2 pnt
@@ -1500,18 +1510,19 @@ k_nl_force_df(const double2 *__restrict__ u, size_t n3, int n_blk,
 
 // planes per z-chunk of a marching stage launch: the caller's choice, else the
 // split with the smallest estimated time.  A chunk restages and re-stencils 2M
-// halo planes and fills its ring (about two planes more); one CTA per SM, so
-// the chunks run in rounds of 152.  (At least 304 CTAs or 16 planes per chunk,
-// the earlier rule, gave 108 CTAs of 24 planes on 16 orbitals of 48^3: 33 us;
-// this gives 144 of 20.)
+// halo planes and fills its ring (about two planes more); CTAs are dealt to 152
+// SMs in rounds, and one CTA alone on an SM runs at about 0.7 of the speed of
+// two.  (At least 304 CTAs or 16 planes per chunk, the earlier rule for one
+// 512-thread CTA per SM, gave 108 CTAs of 24 planes on 16 orbitals of 48^3.)
 inline int stage_zchunk(const OrbLayout &o, int cols) {
   if (o.zchunk > 0) return std::min(o.zchunk, o.n);
   int best = o.n;
-  long cost = 0;
+  double cost = 0.0;
   for (int nz = 1; nz <= std::max(1, o.n / 4); ++nz) {
     const int zc = (o.n + nz - 1) / nz, ctas = cols * ((o.n + zc - 1) / zc);
-    const long c = (long)((ctas + 151) / 152) * (zc + 2 * o.half_order + 2);
-    if (nz == 1 || c < cost) {
+    const double load = (ctas + 151) / 152;
+    const double c = std::max(load, 1.4) * (zc + 2 * o.half_order + 2);
+    if (nz == 1 || c < 0.98 * cost) {
       cost = c;
       best = zc;
     }

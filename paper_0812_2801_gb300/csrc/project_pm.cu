@@ -267,6 +267,8 @@ k_tile_gather(const float2 *__restrict__ u, int n, int nt, int n_orb_pad,
   constexpr int NA = FORCE ? 6 * BO : 2 * BO;
   __shared__ __align__(16) float2 us[512 * BO];
   const int t = blockIdx.x, blk = blockIdx.y;
+  const int S = tile_nat[t];
+  if (S == 0) return;                     // no sphere reaches this tile
   const int tx = t % nt, ty = (t / nt) % nt, tz = t / (nt * nt);
   const size_t n3 = (size_t)n * n * n;
   const float2 *ub = u + (size_t)blk * n3 * BO;
@@ -287,7 +289,6 @@ k_tile_gather(const float2 *__restrict__ u, int n, int nt, int n_orb_pad,
     }
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
-  const int S = tile_nat[t];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int *off = te_off + (size_t)t * (EMD_TILE_ATOM_MAX + 1);
   const size_t tb = (size_t)t * EMD_TE_CAP;
