@@ -393,6 +393,7 @@ void forces(emd_system *s, int k, double field, double dt, int update_v) {
 
 int reduce_max_veff(emd_system *s, double *out);
 double kinetic_fp32(emd_system *s, int *np);
+void kinetic_df(emd_system *s, int *np);
 
 // After new orbitals or ions: rho(0), v_Hxc(0), F(0); history restarts.
 int restart_dynamics(emd_system *s) {
@@ -483,6 +484,28 @@ double kinetic_fp32(emd_system *s, int *np) {
   emd_launch_stage(o, a, s->st);
   emd_launch_cdot_re_c64(s->o, s->psi, s->ua, s->partials, np, s->st);
   return -1.0 / (2.0 * fd_den(order) * s->g.h * s->g.h);
+}
+// complex128, bo = 2: partial sums of Re<psi|T psi>, T psi by the double-float
+// stage (v_eff = 0 in veff1, no projectors) into ua.  The plain FP64 kernel
+// runs ~59 FP64 instructions per point and orbital (13 ms on 96^3 x 128
+// orbitals; this takes 4.5).
+void kinetic_df(emd_system *s, int *np) {
+  cudaMemsetAsync(s->veff1, 0, (size_t)s->g.n3 * sizeof(double), s->st);
+  OrbLayout o = s->o;
+  o.zchunk = 0;
+  StageArgs a;
+  a.u_in = s->psi;
+  a.psi0 = s->psi;
+  a.u_out = s->ua;
+  a.v_eff = s->veff1;
+  a.tab = &s->ts[s->cur];
+  a.err = s->err;
+  a.hc = nullptr;
+  a.a = 0.0;
+  a.apply_only = 1;
+  emd_note_launches(1);
+  emd_launch_stage_df(o, a, s->st);
+  emd_launch_cdot_re_df(s->o, s->psi, s->ua, s->partials, np, s->st);
 }
 int reduce_max_veff(emd_system *s, double *out) {
   emd_note_launches(1);
@@ -655,7 +678,7 @@ int emd_init_system(const emd_config *cfg, emd_system **out) {
     TRY(A((void **)&t.pt_pf, n3 * t.kmax * 4));
     TRY(A((void **)&t.pt4, n3 * 4 * sizeof(int2)));
     TRY(A((void **)&t.at_cnt, na * 4));
-    TRY(A((void **)&t.split_cnt, na * EMD_SPLIT * 4));
+    TRY(A((void **)&t.split_cnt, na * EMD_AT_SPLIT * 4));
     TRY(A((void **)&t.at_pt, (size_t)na * cap * 4));
     TRY(A((void **)&t.at_p, (size_t)na * cap * 8));
     TRY(A((void **)&t.at_d, (size_t)na * cap * 24));
@@ -693,6 +716,13 @@ int emd_init_system(const emd_config *cfg, emd_system **out) {
       TRY(A((void **)&t.gtab, (size_t)na * 27 * 3 * EMD_GT_EXT * sizeof(double)));
       TRY(A((void **)&t.glo, (size_t)na * 27 * 3 * sizeof(int)));
       TRY(A((void **)&t.gtabd, (size_t)na * 27 * EMD_GT_EXT * sizeof(double)));
+    }
+    t.ptab = t.pdtab = nullptr;
+    t.plo = nullptr;
+    if (t.gtab && c.precision == EMD_FP64 && 2 * (int)std::ceil(p.r_proj / c.h) + 6 <= EMD_GT_EXT) {
+      TRY(A((void **)&t.ptab, (size_t)na * 27 * 3 * EMD_GT_EXT * sizeof(double)));
+      TRY(A((void **)&t.pdtab, (size_t)na * 27 * 3 * EMD_GT_EXT * sizeof(double)));
+      TRY(A((void **)&t.plo, (size_t)na * 27 * 3 * sizeof(int)));
     }
     TRY(A((void **)&t.v_loc, n3 * 8));
   }
@@ -1962,6 +1992,8 @@ int emd_get_energy(emd_system *s, emd_energy *out) {
   double kin_scale = 1.0;
   if (s->o.prec == EMD_FP32_ORBITALS)
     kin_scale = kinetic_fp32(s, &np);
+  else if (s->ts[cur].pt4d && s->o.stage_variant != 1)
+    kinetic_df(s, &np);
   else
     emd_launch_kinetic_partials(s->o, s->psi, s->partials, &np, s->st);
   emd_launch_sum(s->partials, np, s->scal + 0, s->st);

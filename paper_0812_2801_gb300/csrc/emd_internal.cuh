@@ -12,7 +12,8 @@
 #define EMD_TE_CAP (EMD_TILE * EMD_TILE * EMD_TILE * EMD_PT_KMAX)
 #define EMD_GT_EXT 64
 #define EMD_SR_SPLIT 8          // CTAs per atom for the short-range ion term
-#define EMD_SPLIT 16            // CTAs per atom for table building and local forces
+#define EMD_SPLIT 16            // CTAs per atom for local forces
+#define EMD_AT_SPLIT 64         // CTAs per atom for the atom-major table
 
 // error bits raised by kernels (device flag, read by emd_get_*)
 // Perdew-Zunger (1981) correlation of the unpolarised uniform gas, the LDA
@@ -107,7 +108,7 @@ struct TableSet {
   // NULL otherwise
   int4 *pt_rec;
   int *at_cnt;      // [n_atoms] (projector P's list: at_cnt[P / n_ch])
-  int *split_cnt;   // [n_atoms][EMD_SPLIT] hits per range (table building)
+  int *split_cnt;   // [n_atoms][EMD_AT_SPLIT] hits per range (table building)
   int *at_pt;       // [n_atoms][cap] flat grid index
   double *at_p;     // [n_atoms][cap] p value of that (point, image)
   double *at_d;     // [n_atoms][cap][3] displacement r - R_image
@@ -141,6 +142,10 @@ struct TableSet {
   double *gtab;
   int *glo;         // [n_atoms][27][3] first grid index of each table
   double *gtabd;    // [n_atoms][27][EMD_GT_EXT] T_x d_x along x
+  // complex128: the same for the projector, exp(-d_a^2 / (2 r_c^2)) along the
+  // image boxes of the r_proj sphere, and the displacements d_a
+  double *ptab, *pdtab;   // [n_atoms][27][3][EMD_GT_EXT]; NULL as for gtab
+  int *plo;               // [n_atoms][27][3]
   double *v_loc;    // [n3] Poisson(-g_ion)
   int cap;
 };
@@ -476,6 +481,7 @@ struct StageArgs {
                                   // FP64, bo = 2: float2, the split diagonal
   const TableSet *tab;
   const void *hc;          // [n_atoms][n_orb_pad] h_kb*c in orbital precision
+                           // (double-float stage: NULL leaves the projectors out)
   double a;                // tau / k ; u_out = psi0 + (-i a) H u_in
   int apply_only;          // 1: u_out = H u_in (psi0 unused)
   int *err = nullptr;      // device error bits (EMD_ERRBIT_*), may be NULL
@@ -597,3 +603,6 @@ void emd_launch_nl_force_tile(const OrbLayout &o, const TableSet &t, int n_atoms
 // per point, FP64 across points)
 void emd_launch_cdot_re_c64(const OrbLayout &o, const void *a, const void *b,
                             double *partials, int *nparts, cudaStream_t st);
+// the same over complex128 arrays with bo = 2
+void emd_launch_cdot_re_df(const OrbLayout &o, const void *a, const void *b, double *partials,
+                           int *nparts, cudaStream_t st);

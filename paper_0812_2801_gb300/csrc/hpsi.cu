@@ -1204,6 +1204,37 @@ __global__ void k_density_df(const double2 *__restrict__ u, size_t n3, int n_blk
   rho[p] = occ * (re + im);
 }
 
+// complex128, bo = 2: the same sum over Re(conj(a) b) with the products and the
+// sum over orbitals in double-float arithmetic (as k_density_df: the real and
+// imaginary products accumulate as packed pairs, TwoProduct of the high parts
+// and the two cross terms, relative error ~1e-14 per point), widened once per
+// point and added in FP64 across points.
+__global__ void __launch_bounds__(256)
+k_cdot_re_df(const double2 *__restrict__ a, const double2 *__restrict__ b, size_t n3, int n_blk,
+             double *part) {
+  __shared__ double red[8];
+  const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  double acc[1] = {0.0};
+  if (p < n3) {
+    float2 ah = make_float2(0.f, 0.f), al = ah;
+#pragma unroll 2
+    for (int k = 0; k < n_blk; ++k) {
+      const size_t o = ((size_t)k * n3 + p) * 2;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const float4 x = df_split2(a[o + j]), y = df_split2(b[o + j]);
+        float2 q, e;
+        dfp_two_prod(f4hi(x), f4hi(y), q, e);
+        dfp_add(ah, al, q, __ffma2_rn(f4hi(x), f4lo(y), __ffma2_rn(f4lo(x), f4hi(y), e)));
+      }
+    }
+    acc[0] = __dadd_rn(__dadd_rn(df_widen(ah.x), df_widen(al.x)),
+                       __dadd_rn(df_widen(ah.y), df_widen(al.y)));
+  }
+  emd_block_sum<1>(acc, red);
+  if (threadIdx.x == 0) part[blockIdx.x] = acc[0];
+}
+
 // partial[b] = sum over the points of block b and all orbitals of
 // Re(conj(u) (-1/2 nabla^2_FD u)), FP64.
 template <typename T, int BO, int M>
@@ -1971,4 +2002,12 @@ void emd_launch_cdot_re_c64(const OrbLayout &o, const void *a, const void *b,
     case 2: k_cdot_re_c64<2><<<nb, 256, 0, st>>>((const float2 *)a, (const float2 *)b, (size_t)o.n3, o.n_blk, partials); break;
     case 4: k_cdot_re_c64<4><<<nb, 256, 0, st>>>((const float2 *)a, (const float2 *)b, (size_t)o.n3, o.n_blk, partials); break;
   }
+}
+
+void emd_launch_cdot_re_df(const OrbLayout &o, const void *a, const void *b, double *partials,
+                           int *nparts, cudaStream_t st) {
+  emd_note_launches(1);
+  *nparts = (o.n3 + 255) / 256;
+  k_cdot_re_df<<<*nparts, 256, 0, st>>>((const double2 *)a, (const double2 *)b, (size_t)o.n3,
+                                        o.n_blk, partials);
 }

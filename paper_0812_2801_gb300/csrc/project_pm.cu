@@ -32,24 +32,33 @@ __global__ void k_tile_atoms(const int *tile_cnt, const int *tile_ent, int ntile
 }
 
 // exclusive prefix sum of tile_nat (one CTA, fixed order) -> tile_off
-__global__ void k_tile_offsets(const int *tile_nat, int ntiles, int *tile_off) {
-  __shared__ int part[1024];
+__global__ void __launch_bounds__(1024)
+k_tile_offsets(const int *tile_nat, int ntiles, int *tile_off) {
+  __shared__ int wsum[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int per = (ntiles + blockDim.x - 1) / blockDim.x;
   const int t0 = threadIdx.x * per, t1 = min(ntiles, t0 + per);
   int s = 0;
   for (int t = t0; t < t1; ++t) s += tile_nat[t];
-  part[threadIdx.x] = s;
+  int x = s;                               // inclusive scan over the warp
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) wsum[warp] = x;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int i = 0; i < (int)blockDim.x; ++i) {
-      const int v = part[i];
-      part[i] = acc;
-      acc += v;
+  if (warp == 0) {                         // and over the warps
+    int w = wsum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += y;
     }
+    wsum[lane] = w;
   }
   __syncthreads();
-  int acc = part[threadIdx.x];
+  int acc = x - s + (warp ? wsum[warp - 1] : 0);
   for (int t = t0; t < t1; ++t) {
     tile_off[t] = acc;
     acc += tile_nat[t];

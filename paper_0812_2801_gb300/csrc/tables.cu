@@ -102,8 +102,8 @@ template <bool F32>
 __global__ void __launch_bounds__(512)
 k_point_table(int n, int n3, double h, double L, const double *Rw,
               SpeciesDev sp, float margin, const int *tile_cnt, const int *tile_ent,
-              const double *gtab, const int *glo,
-              int *pt_cnt, int *pt_J, double *pt_p, float *pt_pf, int2 *pt4, int4 *pt4d,
+              const double *gtab, const int *glo, const double *ptab, const double *pdtab,
+              const int *plo, int *pt_cnt, int *pt_J, double *pt_p, float *pt_pf, int2 *pt4, int4 *pt4d,
               double *g_ion, int *te_off, uint2 *te_pp, float4 *te_q, int kmax, int4 *pt_rec,
               int *err) {
   __shared__ int cand[EMD_TILE_CAND_MAX];
@@ -257,7 +257,27 @@ k_point_table(int n, int n3, double h, double L, const double *Rw,
           g_tab = true;
         }
       }
-      if (!have64 && ((in_l && !g_tab) || (in_p && !F32))) {
+      // and the projector's (complex128)
+      bool p_tab = false;
+      double p_exp = 0.0;
+      if (!F32 && in_p && ptab) {
+        const int *lo = plo + ((size_t)J * 27 + img) * 3;
+        const int kx = x - lo[0], ky = y - lo[1], kz = z - lo[2];
+        if (kx >= 0 && ky >= 0 && kz >= 0 && kx < EMD_GT_EXT && ky < EMD_GT_EXT &&
+            kz < EMD_GT_EXT) {
+          const size_t o = ((size_t)J * 27 + img) * 3 * EMD_GT_EXT;
+          const double *T = ptab + o;
+          p_exp = T[kx] * (T[EMD_GT_EXT + ky] * T[2 * EMD_GT_EXT + kz]);
+          p_tab = true;
+          if (sp.nch > 1 && !have64) {
+            const double *D = pdtab + o;
+            dx = D[kx];
+            dy = D[EMD_GT_EXT + ky];
+            dz = D[2 * EMD_GT_EXT + kz];
+          }
+        }
+      }
+      if (!have64 && ((in_l && !g_tab) || (in_p && !F32 && !p_tab))) {
         dx = emd_disp(x, h, Rw[3 * J + 0], img % 3 - 1, L);
         dy = emd_disp(y, h, Rw[3 * J + 1], (img / 3) % 3 - 1, L);
         dz = emd_disp(z, h, Rw[3 * J + 2], img / 9 - 1, L);
@@ -283,7 +303,7 @@ k_point_table(int n, int n3, double h, double L, const double *Rw,
           pdy += w * ey;
           pdz += w * ez;
         } else {
-          const double ex = exp(-d2 * sp.inv_2rc2);
+          const double ex = p_tab ? p_exp : exp(-d2 * sp.inv_2rc2);
           psum += sp.c_p * ex;
           if (sp.nch > 1) {
             double pk[9];
@@ -411,8 +431,8 @@ __device__ void image_boxes(const double *c, double L, double h, double r,
 // only (the complex64 kernels read the per-tile entries of the point table).
 __global__ void __launch_bounds__(256)
 k_atom_table(int pass, int n, double h, double L, const double *Rw,
-             SpeciesDev sp, int cap, float margin, int *split_cnt, int *at_cnt,
-             int *at_pt, double *at_p, double *at_d, uint4 *at_rec, float4 *at_w,
+             SpeciesDev sp, int cap, float margin, const double *ptab, const double *pdtab,
+             int *split_cnt, int *at_cnt, int *at_pt, double *at_p, double *at_d, uint4 *at_rec, float4 *at_w,
              int *err) {
   __shared__ ImageBoxes B;
   __shared__ float cf[27][3];
@@ -480,11 +500,22 @@ k_atom_table(int pass, int n, double h, double L, const double *Rw,
         const size_t q = (size_t)J * cap + e;
         const int pidx = (iz * n + iy) * n + ix;
         at_pt[q] = pidx;
-        const int ni[3] = {img % 3 - 1, (img / 3) % 3 - 1, img / 9 - 1};
-        const double dx = emd_disp(ix, h, c[0], ni[0], L);
-        const double dy = emd_disp(iy, h, c[1], ni[1], L);
-        const double dz = emd_disp(iz, h, c[2], ni[2], L);
-        const double ex = exp(-emd_norm2(dx, dy, dz) * sp.inv_2rc2);
+        double dx, dy, dz, ex;
+        if (ptab) {                        // this box's 1-D tables
+          const size_t o = ((size_t)J * 27 + img) * 3 * EMD_GT_EXT;
+          const int kx = ix - B.lo[img][0], ky = EMD_GT_EXT + iy - B.lo[img][1],
+                    kz = 2 * EMD_GT_EXT + iz - B.lo[img][2];
+          dx = pdtab[o + kx];
+          dy = pdtab[o + ky];
+          dz = pdtab[o + kz];
+          ex = ptab[o + kx] * (ptab[o + ky] * ptab[o + kz]);
+        } else {
+          const int ni[3] = {img % 3 - 1, (img / 3) % 3 - 1, img / 9 - 1};
+          dx = emd_disp(ix, h, c[0], ni[0], L);
+          dy = emd_disp(iy, h, c[1], ni[1], L);
+          dz = emd_disp(iz, h, c[2], ni[2], L);
+          ex = exp(-emd_norm2(dx, dy, dz) * sp.inv_2rc2);
+        }
         const double pv = sp.c_p * ex;
         at_p[q] = pv;
         double *dd = at_d + 3 * q;
@@ -525,30 +556,40 @@ k_atom_table(int pass, int n, double h, double L, const double *Rw,
   }
 }
 
-// 1-D factors of the ion Gaussian along each image box of atom J's r_loc
-// sphere: exp(-d^2 / a^2) with d the FP64 displacement of grid index
-// lo + i (the same operations as every displacement here), so that
-// g = c_g T_x T_y T_z (three roundings from exp(-|d|^2 / a^2)).  One block
-// per atom.
+// 1-D factors of a Gaussian along each image box of atom J's sphere: exp(-d^2
+// w) with d the FP64 displacement of grid index lo + i (the same operations
+// as every displacement here).  Set 0: the ion Gaussian (w = 1 / a^2, r_loc),
+// g = c_g T_x T_y T_z; set 1: the projector (w = 1 / (2 r_c^2), r_proj), p =
+// c_p T_x T_y T_z (three roundings; the argument of a single exp(-|d|^2 w)
+// rounds at up to |d|^2 w = 12 times that).  Block (atom, axis, set).  gtabd:
+// T d, x axis of set 0; pdtab: d, every axis of set 1.
 __global__ void __launch_bounds__(256)
 k_gauss_tables(int n, double h, double L, const double *Rw, SpeciesDev sp, double *gtab,
-               double *gtabd, int *glo) {
+               double *gtabd, int *glo, double *ptab, double *pdtab, int *plo) {
   __shared__ ImageBoxes B;
-  const int J = blockIdx.x;
+  const int J = blockIdx.x, a = blockIdx.y, set = blockIdx.z;
   const double c[3] = {Rw[3 * J], Rw[3 * J + 1], Rw[3 * J + 2]};
-  image_boxes(c, L, h, sp.r_loc, n, B);
+  image_boxes(c, L, h, set ? sp.r_proj : sp.r_loc, n, B);
   __syncthreads();
-  if (threadIdx.x < 81)
-    glo[(size_t)J * 81 + threadIdx.x] = B.lo[threadIdx.x / 3][threadIdx.x % 3];
-  double *T = gtab + (size_t)J * 27 * 3 * EMD_GT_EXT;
-  for (int q = threadIdx.x; q < 27 * 3 * EMD_GT_EXT; q += blockDim.x) {
-    const int img = q / (3 * EMD_GT_EXT), a = (q / EMD_GT_EXT) % 3, i = q % EMD_GT_EXT;
+  int *lo = set ? plo : glo;
+  if (a == 0 && threadIdx.x < 81)
+    lo[(size_t)J * 81 + threadIdx.x] = B.lo[threadIdx.x / 3][threadIdx.x % 3];
+  const size_t o = (size_t)J * 27 * 3 * EMD_GT_EXT;
+  const double w = set ? sp.inv_2rc2 : sp.inv_a2;
+  for (int q = threadIdx.x; q < 27 * EMD_GT_EXT; q += blockDim.x) {
+    const int img = q / EMD_GT_EXT, i = q % EMD_GT_EXT;
     if (i >= B.ext[img][a] || B.start[img + 1] == B.start[img]) continue;
     const int ni = a == 0 ? img % 3 - 1 : a == 1 ? (img / 3) % 3 - 1 : img / 9 - 1;
     const double d = emd_disp(B.lo[img][a] + i, h, c[a], ni, L);
-    const double t = exp(-__dmul_rn(d, d) * sp.inv_a2);
-    T[q] = t;
-    if (a == 0) gtabd[((size_t)J * 27 + img) * EMD_GT_EXT + i] = t * d;
+    const double t = exp(-__dmul_rn(d, d) * w);
+    const size_t k = o + (size_t)(img * 3 + a) * EMD_GT_EXT + i;
+    if (set) {
+      ptab[k] = t;
+      pdtab[k] = d;
+    } else {
+      gtab[k] = t;
+      if (a == 0) gtabd[((size_t)J * 27 + img) * EMD_GT_EXT + i] = t * d;
+    }
   }
 }
 
@@ -639,7 +680,7 @@ k_local_force(int n, double h, double L, const double *Rw, const double *gtab,
 __global__ void __launch_bounds__(256)
 k_local_force_rows(int n, double h, double L, const double *Rw, const double *gtab,
                    const double *gtabd, SpeciesDev sp, const double *va,
-                   const double *vb, double *part) {
+                   const double *vb, float margin, double *part) {
   __shared__ ImageBoxes B;
   __shared__ int rstart[28];
   __shared__ float cf[27][3];
@@ -670,7 +711,8 @@ k_local_force_rows(int n, double h, double L, const double *Rw, const double *gt
   const int q0 = split * per, q1 = min(nrows, q0 + per);
   double acc[3] = {0.0, 0.0, 0.0};
   int img = 0;
-  for (int q = q0 + threadIdx.x; q < q1; q += blockDim.x) {
+  const int sub = threadIdx.x & 3;                  // four threads per row
+  for (int q = q0 + (threadIdx.x >> 2); q < q1; q += blockDim.x >> 2) {
     while (img < 26 && q >= rstart[img + 1]) ++img;
     const int k = q - rstart[img];
     const int ey = B.ext[img][1];
@@ -688,7 +730,12 @@ k_local_force_rows(int n, double h, double L, const double *Rw, const double *gt
     const int xb = min(hi0, (int)floorf((cf[img][0] + wf) * ihf) + 2);
     const double dy = emd_disp(iy, h, c[1], ni[1], L);
     const double dz = emd_disp(iz, h, c[2], ni[2], L);
+    // in FP32 where it is certain, in FP64 in the shell
+    const float yz2 = dyf * dyf + dzf * dzf;
     auto inside = [&](int x) {
+      const float dxf = (float)x * hf - cf[img][0], d2f = dxf * dxf + yz2;
+      if (d2f < rl2f - margin) return true;
+      if (d2f > rl2f + margin) return false;
       return emd_norm2(emd_disp(x, h, c[0], ni[0], L), dy, dz) < rl2;
     };
     int xs = xa;
@@ -701,7 +748,7 @@ k_local_force_rows(int n, double h, double L, const double *Rw, const double *gt
     const double tyz = Tx[EMD_GT_EXT + ky] * Tx[2 * EMD_GT_EXT + kz];
     const size_t rowp = ((size_t)iz * n + iy) * n;
     double s0 = 0.0, s1 = 0.0;
-    for (int x = xs; x <= xe; ++x) {
+    for (int x = xs + sub; x <= xe; x += 4) {
       const double v = va[rowp + x] + vb[rowp + x];
       s0 += v * Tx[x - lo0];
       s1 += v * Dx[x - lo0];
@@ -824,29 +871,31 @@ void emd_launch_tables(const GridInfo &g, const SpeciesDev &sp, int n_atoms,
       g.n, g.h, g.L, t.Rw, n_atoms, rmax, t.tile_cnt, t.tile_ent, err);
   if (t.gtab && n_atoms > 0) {
     emd_note_launches(1);
-    k_gauss_tables<<<n_atoms, 256, 0, st>>>(g.n, g.h, g.L, t.Rw, sp, t.gtab, t.gtabd,
-                                            t.glo);
+    k_gauss_tables<<<dim3(n_atoms, 3, t.ptab ? 2 : 1), 256, 0, st>>>(
+        g.n, g.h, g.L, t.Rw, sp, t.gtab, t.gtabd, t.glo, t.ptab, t.pdtab, t.plo);
   }
   const float margin_pt = emd_fp32_d2_margin(g.L, fmax(sp.r_proj, sp.r_loc));
   if (t.te_off)
     k_point_table<true><<<ntiles, 512, 0, st>>>(g.n, g.n3, g.h, g.L, t.Rw, sp, margin_pt,
-                                                t.tile_cnt, t.tile_ent, t.gtab, t.glo,
+                                                t.tile_cnt, t.tile_ent, t.gtab, t.glo, t.ptab,
+                                                t.pdtab, t.plo,
                                                 t.pt_cnt, t.pt_J, t.pt_p, t.pt_pf, t.pt4, t.pt4d,
                                                 t.g_ion, t.te_off, t.te_pp, t.te_q,
                                                 t.kmax, nullptr, err);
   else
     k_point_table<false><<<ntiles, 512, 0, st>>>(g.n, g.n3, g.h, g.L, t.Rw, sp, margin_pt,
-                                                 t.tile_cnt, t.tile_ent, t.gtab, t.glo,
+                                                 t.tile_cnt, t.tile_ent, t.gtab, t.glo, t.ptab,
+                                                t.pdtab, t.plo,
                                                  t.pt_cnt, t.pt_J, t.pt_p, t.pt_pf, t.pt4, t.pt4d,
                                                  t.g_ion, t.te_off, t.te_pp, t.te_q,
                                                  t.kmax, t.pt_rec, err);
   if (n_atoms > 0 && !t.te_off) {
-    dim3 grid(n_atoms, EMD_SPLIT);
+    dim3 grid(n_atoms, EMD_AT_SPLIT);
     const float margin = emd_fp32_d2_margin(g.L, sp.r_proj);
     for (int pass = 0; pass < 2; ++pass)
       k_atom_table<<<grid, 256, 0, st>>>(pass, g.n, g.h, g.L, t.Rw, sp, t.cap, margin,
-                                         t.split_cnt, t.at_cnt, t.at_pt, t.at_p, t.at_d,
-                                         t.at_rec, t.at_w, err);
+                                         t.ptab, t.pdtab, t.split_cnt, t.at_cnt, t.at_pt,
+                                         t.at_p, t.at_d, t.at_rec, t.at_w, err);
   }
 }
 
@@ -859,7 +908,8 @@ void emd_launch_local_force(const GridInfo &g, const SpeciesDev &sp,
   dim3 grid(n_atoms, EMD_SPLIT);
   if (t.gtab)
     k_local_force_rows<<<grid, 256, 0, st>>>(g.n, g.h, g.L, t.Rw, t.gtab, t.gtabd, sp,
-                                             v_es_a, v_es_b, part);
+                                             v_es_a, v_es_b,
+                                             emd_fp32_d2_margin(g.L, sp.r_loc), part);
   else
     k_local_force<false><<<grid, 256, 0, st>>>(g.n, g.h, g.L, t.Rw, t.gtab, sp,
                                                emd_fp32_d2_margin(g.L, sp.r_loc), v_es_a,
