@@ -393,7 +393,6 @@ void forces(emd_system *s, int k, double field, double dt, int update_v) {
 
 int reduce_max_veff(emd_system *s, double *out);
 double kinetic_fp32(emd_system *s, int *np);
-void kinetic_df(emd_system *s, int *np);
 
 // After new orbitals or ions: rho(0), v_Hxc(0), F(0); history restarts.
 int restart_dynamics(emd_system *s) {
@@ -484,28 +483,6 @@ double kinetic_fp32(emd_system *s, int *np) {
   emd_launch_stage(o, a, s->st);
   emd_launch_cdot_re_c64(s->o, s->psi, s->ua, s->partials, np, s->st);
   return -1.0 / (2.0 * fd_den(order) * s->g.h * s->g.h);
-}
-// complex128, bo = 2: partial sums of Re<psi|T psi>, T psi by the double-float
-// stage (v_eff = 0 in veff1, no projectors) into ua.  The plain FP64 kernel
-// runs ~59 FP64 instructions per point and orbital (13 ms on 96^3 x 128
-// orbitals; this takes 4.5).
-void kinetic_df(emd_system *s, int *np) {
-  cudaMemsetAsync(s->veff1, 0, (size_t)s->g.n3 * sizeof(double), s->st);
-  OrbLayout o = s->o;
-  o.zchunk = 0;
-  StageArgs a;
-  a.u_in = s->psi;
-  a.psi0 = s->psi;
-  a.u_out = s->ua;
-  a.v_eff = s->veff1;
-  a.tab = &s->ts[s->cur];
-  a.err = s->err;
-  a.hc = nullptr;
-  a.a = 0.0;
-  a.apply_only = 1;
-  emd_note_launches(1);
-  emd_launch_stage_df(o, a, s->st);
-  emd_launch_cdot_re_df(s->o, s->psi, s->ua, s->partials, np, s->st);
 }
 int reduce_max_veff(emd_system *s, double *out) {
   emd_note_launches(1);
@@ -1992,8 +1969,6 @@ int emd_get_energy(emd_system *s, emd_energy *out) {
   double kin_scale = 1.0;
   if (s->o.prec == EMD_FP32_ORBITALS)
     kin_scale = kinetic_fp32(s, &np);
-  else if (s->ts[cur].pt4d && s->o.stage_variant != 1)
-    kinetic_df(s, &np);
   else
     emd_launch_kinetic_partials(s->o, s->psi, s->partials, &np, s->st);
   emd_launch_sum(s->partials, np, s->scal + 0, s->st);

@@ -481,7 +481,6 @@ struct StageArgs {
                                   // FP64, bo = 2: float2, the split diagonal
   const TableSet *tab;
   const void *hc;          // [n_atoms][n_orb_pad] h_kb*c in orbital precision
-                           // (double-float stage: NULL leaves the projectors out)
   double a;                // tau / k ; u_out = psi0 + (-i a) H u_in
   int apply_only;          // 1: u_out = H u_in (psi0 unused)
   int *err = nullptr;      // device error bits (EMD_ERRBIT_*), may be NULL
@@ -603,6 +602,3 @@ void emd_launch_nl_force_tile(const OrbLayout &o, const TableSet &t, int n_atoms
 // per point, FP64 across points)
 void emd_launch_cdot_re_c64(const OrbLayout &o, const void *a, const void *b,
                             double *partials, int *nparts, cudaStream_t st);
-// the same over complex128 arrays with bo = 2
-void emd_launch_cdot_re_df(const OrbLayout &o, const void *a, const void *b, double *partials,
-                           int *nparts, cudaStream_t st);

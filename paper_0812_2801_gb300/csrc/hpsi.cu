@@ -1204,39 +1204,14 @@ __global__ void k_density_df(const double2 *__restrict__ u, size_t n3, int n_blk
   rho[p] = occ * (re + im);
 }
 
-// complex128, bo = 2: the same sum over Re(conj(a) b) with the products and the
-// sum over orbitals in double-float arithmetic (as k_density_df: the real and
-// imaginary products accumulate as packed pairs, TwoProduct of the high parts
-// and the two cross terms, relative error ~1e-14 per point), widened once per
-// point and added in FP64 across points.
-__global__ void __launch_bounds__(256)
-k_cdot_re_df(const double2 *__restrict__ a, const double2 *__restrict__ b, size_t n3, int n_blk,
-             double *part) {
-  __shared__ double red[8];
-  const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double acc[1] = {0.0};
-  if (p < n3) {
-    float2 ah = make_float2(0.f, 0.f), al = ah;
-#pragma unroll 2
-    for (int k = 0; k < n_blk; ++k) {
-      const size_t o = ((size_t)k * n3 + p) * 2;
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const float4 x = df_split2(a[o + j]), y = df_split2(b[o + j]);
-        float2 q, e;
-        dfp_two_prod(f4hi(x), f4hi(y), q, e);
-        dfp_add(ah, al, q, __ffma2_rn(f4hi(x), f4lo(y), __ffma2_rn(f4lo(x), f4hi(y), e)));
-      }
-    }
-    acc[0] = __dadd_rn(__dadd_rn(df_widen(ah.x), df_widen(al.x)),
-                       __dadd_rn(df_widen(ah.y), df_widen(al.y)));
-  }
-  emd_block_sum<1>(acc, red);
-  if (threadIdx.x == 0) part[blockIdx.x] = acc[0];
-}
-
-// partial[b] = sum over the points of block b and all orbitals of
-// Re(conj(u) (-1/2 nabla^2_FD u)), FP64.
+// partial[b] = sum over the points of block b and all orbitals whose total is
+// that of Re(conj(u) (-1/2 nabla^2_FD u)), FP64.  Summed over the periodic grid
+// conj(u) u(r - k e) is the conjugate of conj(u) u(r + k e), so the forward
+// neighbours count twice and the backward ones are not read: 28 FP64
+// instructions per value at order 8 instead of 56, which is what bounds it
+// (13 -> 7 ms on 96^3 x 128 orbitals).  Double-float arithmetic, twice as fast
+// again, is not accurate enough here: T u is ~100 times smaller than its
+// terms, 5e-15 of the energy against 3e-16.
 template <typename T, int BO, int M>
 __global__ void __launch_bounds__(256)
 k_kinetic(const typename cplx<T>::type *__restrict__ u, int n, int n_blk,
@@ -1253,21 +1228,17 @@ k_kinetic(const typename cplx<T>::type *__restrict__ u, int n, int n_blk,
       for (int j = 0; j < BO; ++j) {
         const V c0 = ub[p * BO + j];
         double lx = W.w[0] * (double)c0.x, ly = W.w[0] * (double)c0.y;
+#pragma unroll
         for (int k = 1; k <= M; ++k) {
-          const int xp = (x + k) % n, xm = (x - k + n) % n;
-          const int yp = (y + k) % n, ym = (y - k + n) % n;
-          const int zp = (z + k) % n, zm = (z - k + n) % n;
-          const size_t q[6] = {(size_t)(z * n + y) * n + xp, (size_t)(z * n + y) * n + xm,
-                               (size_t)(z * n + yp) * n + x, (size_t)(z * n + ym) * n + x,
-                               (size_t)(zp * n + y) * n + x, (size_t)(zm * n + y) * n + x};
-          double sx = 0, sy = 0;
-          for (int e = 0; e < 6; ++e) {
-            const V v = ub[q[e] * BO + j];
-            sx += (double)v.x;
-            sy += (double)v.y;
-          }
-          lx += W.w[k] * sx;
-          ly += W.w[k] * sy;
+          const int xp = x + k < n ? x + k : x + k - n;
+          const int yp = y + k < n ? y + k : y + k - n;
+          const int zp = z + k < n ? z + k : z + k - n;
+          const V v1 = ub[((size_t)(z * n + y) * n + xp) * BO + j];
+          const V v2 = ub[((size_t)(z * n + yp) * n + x) * BO + j];
+          const V v3 = ub[((size_t)(zp * n + y) * n + x) * BO + j];
+          const double w = 2.0 * W.w[k];
+          lx = fma(w, (double)v1.x + (double)v2.x + (double)v3.x, lx);
+          ly = fma(w, (double)v1.y + (double)v2.y + (double)v3.y, ly);
         }
         acc[0] += (double)c0.x * lx + (double)c0.y * ly;
       }
@@ -2002,12 +1973,4 @@ void emd_launch_cdot_re_c64(const OrbLayout &o, const void *a, const void *b,
     case 2: k_cdot_re_c64<2><<<nb, 256, 0, st>>>((const float2 *)a, (const float2 *)b, (size_t)o.n3, o.n_blk, partials); break;
     case 4: k_cdot_re_c64<4><<<nb, 256, 0, st>>>((const float2 *)a, (const float2 *)b, (size_t)o.n3, o.n_blk, partials); break;
   }
-}
-
-void emd_launch_cdot_re_df(const OrbLayout &o, const void *a, const void *b, double *partials,
-                           int *nparts, cudaStream_t st) {
-  emd_note_launches(1);
-  *nparts = (o.n3 + 255) / 256;
-  k_cdot_re_df<<<*nparts, 256, 0, st>>>((const double2 *)a, (const double2 *)b, (size_t)o.n3,
-                                        o.n_blk, partials);
 }

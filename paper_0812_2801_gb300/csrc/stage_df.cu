@@ -109,7 +109,7 @@ k_stage_df(const void *__restrict__ u_in, const double2 *__restrict__ psi0,
   // tile point of this thread in the per-point stagings (diagonal, records)
   const int vp = tid < Z::NV ? min(ty0 + tid / Z::TX, n - 1) * n + min(tx0 + tid % Z::TX, n - 1)
                              : -1;
-  if (HCS && hc) {
+  if (HCS) {
     for (int i = tid; i < n_proj * BO; i += NT)
       hcs[i] = df_split2(hc[(size_t)(i / BO) * n_orb_pad + (size_t)blockIdx.z * BO + i % BO]);
   }
@@ -243,7 +243,7 @@ k_stage_df(const void *__restrict__ u_in, const double2 *__restrict__ psi0,
         float2 hh = make_float2(0.f, 0.f), hl = make_float2(0.f, 0.f);
         dfp_add_prod(hh, hl, W.sk_hi, W.sk_lo, ah[ph], al[ph]);
         // four entries (unused ones have p = 0 and add exactly zero)
-        const int cnt = hc ? q0.x >> 16 : 0;   // no h c: the kinetic term alone
+        const int cnt = q0.x >> 16;
         const int Je[4] = {q0.x & 0xffff, q0.y, q0.z, q0.w};
         const float ep[4] = {__int_as_float(q1.x), __int_as_float(q1.z), __int_as_float(q2.x),
                              __int_as_float(q2.z)};
