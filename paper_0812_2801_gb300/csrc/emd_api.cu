@@ -722,7 +722,7 @@ int emd_init_system(const emd_config *cfg, emd_system **out) {
   TRY(A((void **)&s->e_sr, na * 8));
   TRY(A((void **)&s->sr_part, (size_t)na * EMD_SR_SPLIT * 4 * 8));
   TRY(A((void **)&s->nl_part, (size_t)nproj * o.n_blk * 3 * 8));
-  TRY(A((void **)&s->lf_part, (size_t)na * EMD_SPLIT * 3 * 8));
+  TRY(A((void **)&s->lf_part, (size_t)na * EMD_SPLIT_MAX * 3 * 8));
   s->n_partials = std::max(1024, (int)((n3 + 255) / 256));
   TRY(A((void **)&s->partials, (size_t)s->n_partials * 8));
   TRY(A((void **)&s->scal, 16 * 8));

@@ -13,6 +13,7 @@
 #define EMD_GT_EXT 64
 #define EMD_SR_SPLIT 8          // CTAs per atom for the short-range ion term
 #define EMD_SPLIT 16            // CTAs per atom for local forces
+#define EMD_SPLIT_MAX 64        // (few atoms; k_local_force_rows)
 #define EMD_AT_SPLIT 64         // CTAs per atom for the atom-major table
 
 // error bits raised by kernels (device flag, read by emd_get_*)
@@ -455,7 +456,7 @@ void emd_launch_absdiff_partials(int n3, const double *a, const double *b, doubl
 // X + i n3; complex128 for EMD_FP64, complex64 otherwise): G = scale X^H Y
 // (m x m, column-major FP64, summed in FP64 in a fixed order; part holds
 // emd_gram_scratch(n3, m) double2), and B = X V (V column-major FP64)
-int emd_gram_chunks(int n3);
+int emd_gram_chunks(int n3, int m);
 size_t emd_gram_scratch(int n3, int m);
 void emd_launch_gram(int prec, const void *X, const void *Y, int n3, int m, double scale,
                      double2 *part, double2 *G, cudaStream_t st);

@@ -144,7 +144,10 @@ k_gram(const C *__restrict__ X, const C *__restrict__ Y, int n3, int m, int rows
       ys[r][c] = oky ? Y[(size_t)(j0 + c) * n3 + rb + r] : zero;
     }
     __syncthreads();
-    if (sizeof(C) == 16) {
+    // a warp holds two columns b; those past m (and the tile's idle half for
+    // small m) have nothing to add
+    if (j0 + (int)(threadIdx.x >> 5) * 2 >= m) {
+    } else if (sizeof(C) == 16) {
       for (int r = 0; r < 32; ++r) {
         const double2 x = GramT<C>::load(&xs[r][a]), y = GramT<C>::load(&ys[r][b]);
         sr = fma(x.x, y.x, fma(x.y, y.y, sr));           // conj(x) y
@@ -167,17 +170,25 @@ k_gram(const C *__restrict__ X, const C *__restrict__ Y, int n3, int m, int rows
     part[((size_t)chunk * m + (j0 + b)) * m + i0 + a] = make_double2(sr, si);
 }
 
-__global__ void k_gram_sum(const double2 *__restrict__ part, int nchunk, int m, double scale,
-                           double2 *__restrict__ G) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// one warp per entry of G: lane l adds the chunks l, l + 32, ..., then the
+// lanes are added by a fixed tree
+__global__ void __launch_bounds__(256)
+k_gram_sum(const double2 *__restrict__ part, int nchunk, int m, double scale,
+           double2 *__restrict__ G) {
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= m * m) return;
   double sr = 0.0, si = 0.0;
-  for (int c = 0; c < nchunk; ++c) {
+  for (int c = lane; c < nchunk; c += 32) {
     const double2 v = part[(size_t)c * m * m + i];
     sr += v.x;
     si += v.y;
   }
-  G[i] = make_double2(scale * sr, scale * si);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sr += __shfl_xor_sync(0xffffffffu, sr, o);
+    si += __shfl_xor_sync(0xffffffffu, si, o);
+  }
+  if (lane == 0) G[i] = make_double2(scale * sr, scale * si);
 }
 
 // B = X V: X canonical n3 x m, V column-major m x m (FP64), B canonical.
@@ -205,8 +216,10 @@ k_rotate(const C *__restrict__ X, const double2 *__restrict__ V, int n3, int m,
                                             : make_double2(0.0, 0.0);
     }
     __syncthreads();
+    // FP64 multiply-adds are the cost: none for k or columns past m
+    const int kn = j0 + 4 * jq < m ? min(16, m - k0) : 0;
 #pragma unroll 4
-    for (int k = 0; k < 16; ++k) {
+    for (int k = 0; k < kn; ++k) {
       const double2 x = xs[k][rr];
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
@@ -268,20 +281,26 @@ void emd_launch_fill_random(int prec, void *canon, size_t n3, int c0, int c1, un
 
 // G = scale X^H Y (m x m, column-major FP64); part: scratch of
 // emd_gram_scratch(n3, m) double2
-int emd_gram_chunks(int n3) { return std::max(1, std::min(64, n3 / 4096)); }
-size_t emd_gram_scratch(int n3, int m) { return (size_t)emd_gram_chunks(n3) * m * m; }
+// row chunks of k_gram: enough CTAs for 16 per SM with the (m / 16)^2 tiles of
+// G, of at least 96 rows each.  (n3 / 4096 chunks left 3 CTAs on 24^3 with 9
+// states: 1.23 ms per product, 80 % of the ground state.)
+int emd_gram_chunks(int n3, int m) {
+  const int tiles = ((m + 15) / 16) * ((m + 15) / 16);
+  return std::max(1, std::min((16 * 152 + tiles - 1) / tiles, n3 / 96));
+}
+size_t emd_gram_scratch(int n3, int m) { return (size_t)emd_gram_chunks(n3, m) * m * m; }
 
 void emd_launch_gram(int prec, const void *X, const void *Y, int n3, int m, double scale,
                      double2 *part, double2 *G, cudaStream_t st) {
   emd_note_launches(2);
-  const int nchunk = emd_gram_chunks(n3);
+  const int nchunk = emd_gram_chunks(n3, m);
   const int rows = (n3 + nchunk - 1) / nchunk;
   const dim3 grid(nchunk, (m + 15) / 16, (m + 15) / 16);
   if (prec == EMD_FP64)
     k_gram<double2><<<grid, 256, 0, st>>>((const double2 *)X, (const double2 *)Y, n3, m, rows, part);
   else
     k_gram<float2><<<grid, 256, 0, st>>>((const float2 *)X, (const float2 *)Y, n3, m, rows, part);
-  k_gram_sum<<<(m * m + 255) / 256, 256, 0, st>>>(part, nchunk, m, scale, G);
+  k_gram_sum<<<(m * m + 7) / 8, 256, 0, st>>>(part, nchunk, m, scale, G);
 }
 
 void emd_launch_rotate(int prec, const void *X, const double2 *V, int n3, int m, void *B,

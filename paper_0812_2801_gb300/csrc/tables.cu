@@ -748,6 +748,7 @@ k_local_force_rows(int n, double h, double L, const double *Rw, const double *gt
     const double tyz = Tx[EMD_GT_EXT + ky] * Tx[2 * EMD_GT_EXT + kz];
     const size_t rowp = ((size_t)iz * n + iy) * n;
     double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
     for (int x = xs + sub; x <= xe; x += 4) {
       const double v = va[rowp + x] + vb[rowp + x];
       s0 += v * Tx[x - lo0];
@@ -905,7 +906,11 @@ void emd_launch_local_force(const GridInfo &g, const SpeciesDev &sp,
                             cudaStream_t st) {
   if (n_atoms <= 0) return;
   emd_note_launches(2);
-  dim3 grid(n_atoms, EMD_SPLIT);
+  // about 4 CTAs per SM: with 16 per atom, 8 atoms left each CTA several
+  // rounds of rows (37 us on 48^3)
+  const int nsplit = !t.gtab || n_atoms >= 38 ? EMD_SPLIT
+                                              : n_atoms <= 9 ? EMD_SPLIT_MAX : 608 / n_atoms;
+  dim3 grid(n_atoms, nsplit);
   if (t.gtab)
     k_local_force_rows<<<grid, 256, 0, st>>>(g.n, g.h, g.L, t.Rw, t.gtab, t.gtabd, sp,
                                              v_es_a, v_es_b,
@@ -915,7 +920,7 @@ void emd_launch_local_force(const GridInfo &g, const SpeciesDev &sp,
                                                emd_fp32_d2_margin(g.L, sp.r_loc), v_es_a,
                                                v_es_b, nullptr, part);
   const int m = 3 * n_atoms;
-  k_local_force_sum<<<(m + 127) / 128, 128, 0, st>>>(part, n_atoms, EMD_SPLIT, F);
+  k_local_force_sum<<<(m + 127) / 128, 128, 0, st>>>(part, n_atoms, nsplit, F);
 }
 
 void emd_launch_local_force_hvp(const GridInfo &g, const SpeciesDev &sp,
