@@ -143,6 +143,7 @@ struct emd_system {
   double2 *c = nullptr;
   void *hc = nullptr;
   int c_valid = 0;
+  int ub_split = 0;               // ub holds the split values of psi (after an MD step)
   double *V = nullptr, *F = nullptr, *F_loc = nullptr, *F_nl = nullptr,
          *F_sr = nullptr, *e_sr = nullptr, *nl_part = nullptr, *lf_part = nullptr,
          *sr_part = nullptr;
@@ -331,21 +332,37 @@ void stage(emd_system *s, const void *u_in, const void *psi0, void *u_out,
   }
 }
 
+// Whether the double-float stage keeps its intermediate sets as split values.
+bool split_sets(const emd_system *s) {
+  return s->veff1s && s->o.stage_variant != 1 && (s->proj_atom_major || s->sp.nch > 1) &&
+         emd_stage_df_splits(s->o);
+}
+
 // One exponential T4(-i tau H) psi0 -> out, H given by (set, veff).
-// Requires hc to hold the projections of psi0 at `set` on entry, and the
-// split diagonal of the potential if the system has one.  The double-float
-// stage keeps the three intermediate sets as split values.
+// Requires hc to hold the projections of psi0 at `set` on entry.
 void exponential(emd_system *s, void *psi0, void *w1, void *out, int set,
                  int which_veff, double tau) {
-  const int sp = s->veff1s && s->o.stage_variant != 1 &&
-                 (s->proj_atom_major || s->sp.nch > 1) && emd_stage_df_splits(s->o);
-  stage(s, psi0, psi0, w1, set, which_veff, tau / 4.0, 0, sp);
-  project(s, w1, set, s->st, sp);
-  stage(s, w1, psi0, out, set, which_veff, tau / 3.0, sp, sp);
-  project(s, out, set, s->st, sp);
-  stage(s, out, psi0, w1, set, which_veff, tau / 2.0, sp, sp);
-  project(s, w1, set, s->st, sp);
-  stage(s, w1, psi0, out, set, which_veff, tau, sp, 0);
+  stage(s, psi0, psi0, w1, set, which_veff, tau / 4.0);
+  project(s, w1, set);
+  stage(s, w1, psi0, out, set, which_veff, tau / 3.0);
+  project(s, out, set);
+  stage(s, out, psi0, w1, set, which_veff, tau / 2.0);
+  project(s, w1, set);
+  stage(s, w1, psi0, out, set, which_veff, tau);
+}
+
+// The same with split intermediate sets (the split diagonal of the potential
+// is in place).  u0: the set that holds psi0's split values, or psi0 itself if
+// there is none.  On return out holds the result and psi0 its split values.
+void exponential_split(emd_system *s, void *u0, void *psi0, void *w1, void *out, int set,
+                       int which_veff, double tau) {
+  stage(s, u0, psi0, w1, set, which_veff, tau / 4.0, u0 != psi0, 1);
+  project(s, w1, set, s->st, true);
+  stage(s, w1, psi0, out, set, which_veff, tau / 3.0, 1, 1);
+  project(s, out, set, s->st, true);
+  stage(s, out, psi0, w1, set, which_veff, tau / 2.0, 1, 1);
+  project(s, w1, set, s->st, true);
+  stage(s, w1, psi0, out, set, which_veff, tau, 1, 2);
 }
 
 // rho, v_H, v_xc of psi into hist slot `slot`.
@@ -852,6 +869,7 @@ static int upload_orbitals_c64(emd_system *s, const float *psi, void *dst) {
 int emd_set_orbitals_c64(emd_system *s, const float *psi) {
   g_err.clear();
   if (!s || !psi) return fail(EMD_EINVAL, "NULL argument");
+  s->ub_split = 0;
   CK(cudaMemsetAsync(s->psi, 0, s->orb_bytes, s->st));
   int r = upload_orbitals_c64(s, psi, s->psi);
   if (r) return r;
@@ -896,6 +914,7 @@ int emd_get_orbitals_c64(emd_system *s, float *psi) {
 int emd_set_orbitals(emd_system *s, const double *psi) {
   g_err.clear();
   if (!s || !psi) return fail(EMD_EINVAL, "NULL argument");
+  s->ub_split = 0;
   CK(cudaMemsetAsync(s->psi, 0, s->orb_bytes, s->st));
   int r = upload_orbitals(s, psi, s->o.n_orb, s->psi);
   if (r) return r;
@@ -916,6 +935,7 @@ int emd_set_occupations(emd_system *s, const double *f) {
   // orbitals already on the device: u_A <- sqrt(f_new / f_old) u_A in two
   // scalings (remove the old weight, apply the new one)
   const int had = s->orbs_set && !s->f_uniform;
+  s->ub_split = 0;
   if (had) emd_launch_scale_orbitals(s->o, s->psi, s->o.n_orb, s->occ_winv, s->st);
   int r = set_occupation_state(s, f);
   if (r) return r;
@@ -1020,19 +1040,28 @@ int step_once(emd_system *s, double dt, double mu, double e) {
   emd_launch_veff(s->g, s->ts[cur].v_loc, s->hist, 1, e, s->veff1, s->veff1f,
                   s->st, s->veff1d, s->o.w[0], s->veff1s, s->o.dv_scale(), s->o.dv_shift());
   if (!s->c_valid) project(s, s->psi, cur);
-  // exponential 1: psi -> ub with H(t)
-  exponential(s, s->psi, s->ua, s->ub, cur, 1, tau);
+  // exponential 1: psi -> ub with H(t); exponential 2: ub -> psi with H(t+dt).
+  // In split form each leaves its result's split values in the set it started
+  // from, which the next one reads and then reuses
+  const bool sp = split_sets(s);
+  if (sp) exponential_split(s, s->ub_split ? s->ub : s->psi, s->psi, s->ua, s->ub, cur, 1, tau);
+  else exponential(s, s->psi, s->ua, s->ub, cur, 1, tau);
   if (!s->frozen_ions) CK(cudaStreamWaitEvent(s->st, s->tev[1], 0));
-  project(s, s->ub, nw);
-  // exponential 2: ub -> psi with H(t+dt)
-  exponential(s, s->ub, s->ua, s->psi, nw, 2, tau);
+  if (sp) {
+    project(s, s->psi, nw, s->st, true);
+    exponential_split(s, s->psi, s->ub, s->ua, s->psi, nw, 2, tau);
+  } else {
+    project(s, s->ub, nw);
+    exponential(s, s->ub, s->ua, s->psi, nw, 2, tau);
+  }
+  s->ub_split = sp;
   if (!s->frozen_ions) {
     // psi's projections at set nw and the nonlocal and short-range forces
     // on the table stream, beside the density and potentials (which they
     // neither read nor write)
     CK(cudaEventRecord(s->tev[0], s->st));
     CK(cudaStreamWaitEvent(s->tst, s->tev[0], 0));
-    project(s, s->psi, nw, s->tst);
+    project(s, sp ? s->ub : s->psi, nw, s->tst, sp);
     forces_nl_sr(s, nw, s->tst);
     CK(cudaEventRecord(s->tev[1], s->tst));
   }
@@ -1235,11 +1264,13 @@ int emd_batch_propagate(emd_batch *b, int n_steps, double dt, double mu) {
       for (size_t i = 0; i < m && rc == EMD_OK; ++i)
         rc = step_once(b->sys[i], dt, mu, 0.0);
   };
-  // a captured chunk assumes the full v_Hxc history and valid projections
-  // of psi (its first step skips re-projecting): step eagerly until both hold
+  // a captured chunk assumes the full v_Hxc history, valid projections of psi
+  // (its first step skips re-projecting) and, in split form, psi's split values
+  // in ub: step eagerly until all hold
   auto full_history = [&]() {
     for (size_t i = 0; i < m; ++i)
-      if (b->sys[i]->hist_len < 3 || b->sys[i]->frozen_ions || !b->sys[i]->c_valid)
+      if (b->sys[i]->hist_len < 3 || b->sys[i]->frozen_ions || !b->sys[i]->c_valid ||
+          b->sys[i]->ub_split != (int)split_sets(b->sys[i]))
         return false;
     return true;
   };
@@ -1589,6 +1620,7 @@ int adjoint_moving(emd_system *s, int n_steps, double dt, double mu,
   int setA = 0;
   for (int ck = n_ck - 1; ck >= 0; --ck) {
     const int n0 = ck * K, n1 = std::min(n_steps, n0 + K);
+    s->ub_split = 0;
     CK(cudaMemcpyAsync(s->psi, A->ck_psi[ck], s->orb_bytes, cudaMemcpyDeviceToDevice, s->st));
     copy_hist_in(s, A->ck_hist[ck]);
     s->hist_len = A->ck_len[ck];
@@ -1717,6 +1749,7 @@ int adjoint_moving(emd_system *s, int n_steps, double dt, double mu,
   std::vector<double> df(n_steps);
   CK(cudaMemcpyAsync(df.data(), A->dfield, n_steps * 8, cudaMemcpyDeviceToHost, s->st));
   // leave the system at the final state
+  s->ub_split = 0;
   CK(cudaMemcpyAsync(s->psi, A->ck_psi[n_ck], s->orb_bytes, cudaMemcpyDeviceToDevice, s->st));
   copy_hist_in(s, A->ck_hist[n_ck]);
   s->hist_len = A->ck_len[n_ck];
@@ -1850,6 +1883,7 @@ int emd_propagate_adjoint(emd_system *s, int n_steps, double dt, double mu,
   // ---- reverse sweep, last segment first
   for (int ck = n_ck - 1; ck >= 0; --ck) {
     const int n0 = ck * K, n1 = std::min(n_steps, n0 + K);
+    s->ub_split = 0;
     CK(cudaMemcpyAsync(s->psi, A->ck_psi[ck], s->orb_bytes, cudaMemcpyDeviceToDevice, s->st));
     copy_hist_in(s, A->ck_hist[ck]);
     s->hist_len = A->ck_len[ck];
@@ -1928,6 +1962,7 @@ int emd_propagate_adjoint(emd_system *s, int n_steps, double dt, double mu,
   if (dL_dfield)
     CK(cudaMemcpyAsync(dL_dfield, A->dfield, n_steps * 8, cudaMemcpyDeviceToHost, s->st));
   // leave the system at the final state
+  s->ub_split = 0;
   CK(cudaMemcpyAsync(s->psi, A->ck_psi[n_ck], s->orb_bytes, cudaMemcpyDeviceToDevice, s->st));
   copy_hist_in(s, A->ck_hist[n_ck]);
   s->hist_len = A->ck_len[n_ck];
@@ -2097,6 +2132,7 @@ int emd_apply_hamiltonian(emd_system *s, int n_vec, const double *psi,
   if (!s->ions_set || !s->orbs_set) return fail(EMD_ESTATE, "set ions and orbitals first");
   int r = ensure_state(s);
   if (r) return r;
+  s->ub_split = 0;                          // ub takes H psi
   CK(cudaMemsetAsync(s->ua, 0, s->orb_bytes, s->st));
   r = upload_orbitals(s, psi, n_vec, s->ua);
   if (r) return r;
@@ -2355,6 +2391,7 @@ int emd_ground_state_smeared(emd_system *s, int max_scf, double tol, int degree,
   constexpr int K = GroundStateWork::kHist;
   s->c_valid = 0;
   s->needs_restart = 1;                     // whatever happens, derived state is stale
+  s->ub_split = 0;
   // starting subspace: the current orbitals (occupation weights removed) and
   // random buffer states; starting density: theirs, scaled to n_e electrons
   gs_unpack(s->o, s->psi, g->B, n_occ, s->st);

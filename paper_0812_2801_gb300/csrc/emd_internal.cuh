@@ -487,7 +487,8 @@ struct StageArgs {
   int *err = nullptr;      // device error bits (EMD_ERRBIT_*), may be NULL
   // complex128, bo = 2: u_in / u_out as split double-float values (float4 (re
   // hi, im hi, re lo, im lo) in place of each double2); in_split needs v_diag,
-  // the split diagonal (float2 per point)
+  // the split diagonal (float2 per point).  out_split = 2 (with in_split):
+  // u_out complex128 and its split values over psi0
   int in_split = 0, out_split = 0;
 };
 struct OrbLayout {

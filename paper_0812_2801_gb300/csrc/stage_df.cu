@@ -17,10 +17,11 @@
 // What bounds it: FP32 issue.  An update at order 8 takes 302 packed FP32x2
 // instructions of two issue cycles each; everything else is kept small:
 //  * u_2, u_3, u_4 live between the stages as split values (16 bytes, like the
-//    complex128 ones), so a value is split once, by the thread that computed
-//    it, instead of by each of the three tiles that stage it and each of the
-//    atoms that project it.  The splits are those that the readers would have
-//    made: the results keep their bits.
+//    complex128 ones), and the last stage leaves its result in both forms, so
+//    a value is split once, by the thread that computed it, instead of by each
+//    of the three tiles that stage it and each of the atoms that project it.
+//    The splits are those that the readers would have made: the results keep
+//    their bits.
 //  * Planes zi that lie in the z halo of the chunk only feed the z direction:
 //    they skip the x/y shells and stage no x/y halo.
 //  * The z direction accumulates in a register line of 2M+1 outputs per
@@ -31,6 +32,10 @@
 // through z; 256 threads, 128 registers, two CTAs per SM, so that one CTA
 // computes while the other waits at its barrier.  Planes arrive by cp.async
 // two ahead in a ring of three.
+// Measured on 96^3 x 128 orbitals, order 8: 4.06 ms per launch before (one CTA
+// of 512 threads, every staged value split by its tile), 2.85-2.90 ms with
+// split input, 3.46 ms with complex128 input (568 instead of 707 instructions
+// per update, FP32 pipe 59 % busy).  32^3 x 16, order 4: 60 -> 22 us.
 #include "emd_internal.cuh"
 
 namespace {
@@ -62,14 +67,19 @@ template <int M> struct DFTile {
 // are read with four in flight); a separate instantiation keeps the
 // s-projector kernel's registers as they were.  IN / OUT: u_in / u_out as
 // split values (float4) instead of complex128; IN reads the split diagonal dv.
-template <int M, bool HCS, bool MP, bool IN, bool OUT>
+// OUT = 2: complex128, and the split values over psi0 (dup): a point of psi0 is
+// staged by the CTA that writes it, two planes before it writes it, and by no
+// other, so the next exponential's first stage reads split values without a
+// further orbital set.
+template <int M, bool HCS, bool MP, bool IN, int OUT>
 __global__ void __launch_bounds__(256, 2)
 k_stage_df(const void *__restrict__ u_in, const double2 *__restrict__ psi0,
            void *__restrict__ u_out, const double *__restrict__ v_eff,
            const float2 *__restrict__ dv, const int4 *__restrict__ pt4d,
            const int *__restrict__ pt_J, const double *__restrict__ pt_p,
            const int4 *__restrict__ pt_rec, const double2 *__restrict__ hc, int n, int ntx,
-           int zc, int n_orb_pad, int n_proj, double a, int apply_only, DFWeights W) {
+           int zc, int n_orb_pad, int n_proj, double a, int apply_only, float4 *dup,
+           DFWeights W) {
   typedef DFTile<M> Z;
   constexpr int BO = Z::BO, NS = Z::NS, SW = Z::SW, NT = Z::NT;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -304,8 +314,9 @@ k_stage_df(const void *__restrict__ u_in, const double2 *__restrict__ psi0,
         }
         if (valid) {
           const size_t o = boff + po * BO + j;
-          if (OUT) static_cast<float4 *>(u_out)[o] = df_split2(out);
+          if (OUT == 1) static_cast<float4 *>(u_out)[o] = df_split2(out);
           else static_cast<double2 *>(u_out)[o] = out;
+          if (OUT == 2) dup[o] = df_split2(out);
         }
       }
     }
@@ -340,7 +351,7 @@ int df_zchunk(const OrbLayout &o, int cols) {
   return best;
 }
 
-template <int M, bool HCS, bool MP, bool IN, bool OUT>
+template <int M, bool HCS, bool MP, bool IN, int OUT>
 void stage_df_tt(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
   typedef DFTile<M> Z;
   const int fixed = 3 * Z::RSLOT + (IN ? 0 : 2 * Z::DSLOT);
@@ -364,16 +375,17 @@ void stage_df_tt(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
   k_stage_df<M, HCS, MP, IN, OUT><<<grid, Z::NT, smem, st>>>(
       a.u_in, (const double2 *)a.psi0, a.u_out, (const double *)a.v_eff,
       (const float2 *)a.v_diag, a.tab->pt4d, a.tab->pt_J, a.tab->pt_p, a.tab->pt_rec,
-      (const double2 *)a.hc, o.n, ntx, zc, o.n_orb_pad, o.n_proj, a.a, a.apply_only, W);
+      (const double2 *)a.hc, o.n, ntx, zc, o.n_orb_pad, o.n_proj, a.a, a.apply_only,
+      OUT == 2 ? (float4 *)a.psi0 : nullptr, W);
 }
 
 template <int M, bool MP>
 void stage_df_t(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
-  if (!emd_stage_df_splits(o)) stage_df_tt<M, false, MP, false, false>(o, a, st);
-  else if (a.in_split && a.out_split) stage_df_tt<M, true, MP, true, true>(o, a, st);
-  else if (a.in_split) stage_df_tt<M, true, MP, true, false>(o, a, st);
-  else if (a.out_split) stage_df_tt<M, true, MP, false, true>(o, a, st);
-  else stage_df_tt<M, true, MP, false, false>(o, a, st);
+  if (!emd_stage_df_splits(o)) stage_df_tt<M, false, MP, false, 0>(o, a, st);
+  else if (a.in_split && a.out_split == 2) stage_df_tt<M, true, MP, true, 2>(o, a, st);
+  else if (a.in_split) stage_df_tt<M, true, MP, true, 1>(o, a, st);
+  else if (a.out_split) stage_df_tt<M, true, MP, false, 1>(o, a, st);
+  else stage_df_tt<M, true, MP, false, 0>(o, a, st);
 }
 
 template <int M>
