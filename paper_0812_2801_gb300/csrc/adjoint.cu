@@ -24,11 +24,12 @@ __global__ void k_axpy(double2 *y, const double2 *x, size_t n) {
   }
 }
 
-// g[p] += b * Im sum_{blk, j} conj(mu) u
+// g[p] += b * Im sum_{blk, j} conj(mu) u, and acc (+)= mu (first: acc = mu):
+// one pass over mu instead of two
 template <int BO>
 __global__ void k_gv_accum(const double2 *__restrict__ mu,
                            const double2 *__restrict__ u, size_t n3, int n_blk,
-                           double b, double *g) {
+                           double b, double *g, double2 *__restrict__ acc, int first) {
   const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n3) return;
   double s = 0.0;
@@ -38,6 +39,8 @@ __global__ void k_gv_accum(const double2 *__restrict__ mu,
     for (int j = 0; j < BO; ++j) {
       const double2 m = mu[o + j], v = u[o + j];
       s += m.x * v.y - m.y * v.x;   // Im(conj(m) v)
+      const double2 a = first ? make_double2(0.0, 0.0) : acc[o + j];
+      acc[o + j] = make_double2(a.x + m.x, a.y + m.y);
     }
   }
   g[p] += b * s;
@@ -238,13 +241,13 @@ void emd_adj_axpy(double2 *y, const double2 *x, size_t n, cudaStream_t st) {
 }
 
 void emd_adj_gv(const OrbLayout &o, const double2 *mu, const double2 *u, double b,
-                double *g, cudaStream_t st) {
+                double *g, double2 *acc, int first, cudaStream_t st) {
   emd_note_launches(1);
   const unsigned nb = (unsigned)((o.n3 + 255) / 256);
   switch (o.bo) {
-    case 1: k_gv_accum<1><<<nb, 256, 0, st>>>(mu, u, (size_t)o.n3, o.n_blk, b, g); break;
-    case 2: k_gv_accum<2><<<nb, 256, 0, st>>>(mu, u, (size_t)o.n3, o.n_blk, b, g); break;
-    case 4: k_gv_accum<4><<<nb, 256, 0, st>>>(mu, u, (size_t)o.n3, o.n_blk, b, g); break;
+    case 1: k_gv_accum<1><<<nb, 256, 0, st>>>(mu, u, (size_t)o.n3, o.n_blk, b, g, acc, first); break;
+    case 2: k_gv_accum<2><<<nb, 256, 0, st>>>(mu, u, (size_t)o.n3, o.n_blk, b, g, acc, first); break;
+    case 4: k_gv_accum<4><<<nb, 256, 0, st>>>(mu, u, (size_t)o.n3, o.n_blk, b, g, acc, first); break;
   }
 }
 

@@ -1455,14 +1455,12 @@ void reverse_exponential(emd_system *s, const double2 *mu_in, double2 *acc,
   const OrbLayout &o = s->o;
   const size_t nel = (size_t)o.n_blk * o.n3 * o.bo;
   const double h3 = s->g.h * s->g.h * s->g.h;
-  double2 *mu = A->mu, *mu2 = A->mu + nel;
-  cudaMemcpyAsync(mu, mu_in, s->orb_bytes, cudaMemcpyDeviceToDevice, s->st);
-  cudaMemsetAsync(acc, 0, s->orb_bytes, s->st);
+  double2 *mu2 = A->mu + nel;
+  const double2 *mu = mu_in;              // then the two halves of A->mu in turn
   const TableSet &t = s->ts[set];
   for (int k = 1; k <= 4; ++k) {
     const double b = tau / k;
-    emd_adj_axpy(acc, mu, nel, s->st);
-    emd_adj_gv(o, mu, u[k - 1], b, gv, s->st);
+    emd_adj_gv(o, mu, u[k - 1], b, gv, acc, k == 1, s->st);
     emd_adj_project_grad(o, t, s->n_atoms, mu, h3, s->sp.h_kb, s->sp.inv_rc2,
                          A->cm, (double2 *)s->hc, A->dcm, s->st);
     emd_adj_project_grad(o, t, s->n_atoms, u[k - 1], h3, s->sp.h_kb,
@@ -1471,7 +1469,8 @@ void reverse_exponential(emd_system *s, const double2 *mu_in, double2 *acc,
                       o.n_orb_pad, s->sp.h_kb * b / h3, gR, s->st);
     // mu <- conj(a_k) H mu = (+i b) H mu
     stage(s, mu, A->zero, mu2, set, which_veff, -b);
-    std::swap(mu, mu2);
+    mu = mu2;
+    mu2 = mu2 == A->mu ? A->mu + nel : A->mu;
   }
   emd_adj_axpy(acc, mu, nel, s->st);
 }

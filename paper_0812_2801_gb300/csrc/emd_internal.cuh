@@ -559,7 +559,7 @@ void emd_launch_project_pm(const OrbLayout &o, const TableSet &t, int n_atoms,
 // adjoint.cu (FP64 orbitals)
 void emd_adj_axpy(double2 *y, const double2 *x, size_t n, cudaStream_t st);
 void emd_adj_gv(const OrbLayout &o, const double2 *mu, const double2 *u, double b,
-                double *g, cudaStream_t st);
+                double *g, double2 *acc, int first, cudaStream_t st);
 void emd_adj_project_grad(const OrbLayout &o, const TableSet &t, int n_atoms,
                           const double2 *x, double h3, double h_kb,
                           double inv_rc2, double2 *c, double2 *hc, double2 *dc,
