@@ -720,12 +720,13 @@ int emd_init_system(const emd_config *cfg, emd_system **out) {
     TRY(A((void **)&t.at_rows, (size_t)na * ntiles * 4));
     TRY(A((void **)&t.g_ion, n3 * 8));
     t.gtab = nullptr;
-    t.glo = nullptr;
+    t.glo = t.gext = nullptr;
     t.gtabd = nullptr;
     // an image box spans at most 2 r / h + 5 points per axis
     if (c.n_atoms > 0 && 2 * (int)std::ceil(p.r_loc / c.h) + 6 <= EMD_GT_EXT) {
       TRY(A((void **)&t.gtab, (size_t)na * 27 * 3 * EMD_GT_EXT * sizeof(double)));
       TRY(A((void **)&t.glo, (size_t)na * 27 * 3 * sizeof(int)));
+      TRY(A((void **)&t.gext, (size_t)na * 27 * 3 * sizeof(int)));
       TRY(A((void **)&t.gtabd, (size_t)na * 27 * EMD_GT_EXT * sizeof(double)));
     }
     t.ptab = t.pdtab = nullptr;

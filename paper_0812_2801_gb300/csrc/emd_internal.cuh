@@ -141,7 +141,7 @@ struct TableSet {
   // the image box of the r_loc sphere, [n_atoms][27][3][EMD_GT_EXT]; NULL if
   // a box is longer than EMD_GT_EXT points (the kernels then call exp)
   double *gtab;
-  int *glo;         // [n_atoms][27][3] first grid index of each table
+  int *glo, *gext;  // [n_atoms][27][3] first grid index of each table, points
   double *gtabd;    // [n_atoms][27][EMD_GT_EXT] T_x d_x along x
   // complex128: the same for the projector, exp(-d_a^2 / (2 r_c^2)) along the
   // image boxes of the r_proj sphere, and the displacements d_a

@@ -565,15 +565,17 @@ k_atom_table(int pass, int n, double h, double L, const double *Rw,
 // T d, x axis of set 0; pdtab: d, every axis of set 1.
 __global__ void __launch_bounds__(256)
 k_gauss_tables(int n, double h, double L, const double *Rw, SpeciesDev sp, double *gtab,
-               double *gtabd, int *glo, double *ptab, double *pdtab, int *plo) {
+               double *gtabd, int *glo, int *gext, double *ptab, double *pdtab, int *plo) {
   __shared__ ImageBoxes B;
   const int J = blockIdx.x, a = blockIdx.y, set = blockIdx.z;
   const double c[3] = {Rw[3 * J], Rw[3 * J + 1], Rw[3 * J + 2]};
   image_boxes(c, L, h, set ? sp.r_proj : sp.r_loc, n, B);
   __syncthreads();
   int *lo = set ? plo : glo;
-  if (a == 0 && threadIdx.x < 81)
+  if (a == 0 && threadIdx.x < 81) {
     lo[(size_t)J * 81 + threadIdx.x] = B.lo[threadIdx.x / 3][threadIdx.x % 3];
+    if (!set) gext[(size_t)J * 81 + threadIdx.x] = B.ext[threadIdx.x / 3][threadIdx.x % 3];
+  }
   const size_t o = (size_t)J * 27 * 3 * EMD_GT_EXT;
   const double w = set ? sp.inv_2rc2 : sp.inv_a2;
   for (int q = threadIdx.x; q < 27 * EMD_GT_EXT; q += blockDim.x) {
@@ -679,29 +681,37 @@ k_local_force(int n, double h, double L, const double *Rw, const double *gtab,
 // from k_gauss_tables.  Used for the forward force when the tables exist.
 __global__ void __launch_bounds__(256)
 k_local_force_rows(int n, double h, double L, const double *Rw, const double *gtab,
-                   const double *gtabd, SpeciesDev sp, const double *va,
-                   const double *vb, float margin, double *part) {
-  __shared__ ImageBoxes B;
+                   const double *gtabd, const int *glo, const int *gext, SpeciesDev sp,
+                   const double *va, const double *vb, float margin, double *part) {
+  // the image boxes come from k_gauss_tables: their FP64 ranges, worked out
+  // again by every CTA, took as long as its rows
+  struct { int lo[27][3], ext[27][3]; } __shared__ B;
   __shared__ int rstart[28];
   __shared__ float cf[27][3];
-  __shared__ double red[8 * 3];
+  __shared__ double red[8 * 4], res[4];
   const int J = blockIdx.x, split = blockIdx.y, nsplit = gridDim.y;
   const double c[3] = {Rw[3 * J], Rw[3 * J + 1], Rw[3 * J + 2]};
   const double rl2 = __dmul_rn(sp.r_loc, sp.r_loc);
   const float rl2f = (float)rl2, hf = (float)h, ihf = (float)(1.0 / h);
-  image_boxes(c, L, h, sp.r_loc, n, B);
-  if (threadIdx.x == 0) {
-    int acc = 0;   // rows (y, z) per image, boxes with no point skipped
-    for (int img = 0; img < 27; ++img) {
-      rstart[img] = acc;
-      if (B.start[img + 1] > B.start[img]) acc += B.ext[img][1] * B.ext[img][2];
-    }
-    rstart[27] = acc;
-  }
   if (threadIdx.x < 81) {
     const int img = threadIdx.x / 3, a = threadIdx.x % 3;
     const int ni = a == 0 ? img % 3 - 1 : a == 1 ? (img / 3) % 3 - 1 : img / 9 - 1;
+    B.lo[img][a] = __ldg(glo + (size_t)J * 81 + threadIdx.x);
+    B.ext[img][a] = __ldg(gext + (size_t)J * 81 + threadIdx.x);
     cf[img][a] = (float)(c[a] + ni * L);
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {   // rows (y, z) per image, boxes with no point skipped
+    const int img = threadIdx.x;
+    const int own = img < 27 && B.ext[img][0] > 0 ? B.ext[img][1] * B.ext[img][2] : 0;
+    int s = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, s, o);
+      if (img >= o) s += y;
+    }
+    if (img < 27) rstart[img] = s - own;
+    if (img == 27) rstart[27] = s;
   }
   __syncthreads();
   const double *TJ = gtab + (size_t)J * 27 * 3 * EMD_GT_EXT;
@@ -709,7 +719,7 @@ k_local_force_rows(int n, double h, double L, const double *Rw, const double *gt
   const int nrows = rstart[27];
   const int per = (nrows + nsplit - 1) / nsplit;
   const int q0 = split * per, q1 = min(nrows, q0 + per);
-  double acc[3] = {0.0, 0.0, 0.0};
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
   int img = 0;
   const int sub = threadIdx.x & 3;                  // four threads per row
   for (int q = q0 + (threadIdx.x >> 2); q < q1; q += blockDim.x >> 2) {
@@ -759,10 +769,10 @@ k_local_force_rows(int n, double h, double L, const double *Rw, const double *gt
     acc[1] += w * dy * s0;
     acc[2] += w * dz * s0;
   }
-  emd_block_sum<3>(acc, red);
-  if (threadIdx.x == 0) {
+  emd_split_sum<4>(acc, red, res, GatherScratch(), 0, 0, 1);
+  if (threadIdx.x < 3) {
     const double h3 = h * h * h;
-    for (int a = 0; a < 3; ++a) part[((size_t)J * nsplit + split) * 3 + a] = h3 * acc[a];
+    part[((size_t)J * nsplit + split) * 3 + threadIdx.x] = h3 * res[threadIdx.x];
   }
 }
 
@@ -873,7 +883,7 @@ void emd_launch_tables(const GridInfo &g, const SpeciesDev &sp, int n_atoms,
   if (t.gtab && n_atoms > 0) {
     emd_note_launches(1);
     k_gauss_tables<<<dim3(n_atoms, 3, t.ptab ? 2 : 1), 256, 0, st>>>(
-        g.n, g.h, g.L, t.Rw, sp, t.gtab, t.gtabd, t.glo, t.ptab, t.pdtab, t.plo);
+        g.n, g.h, g.L, t.Rw, sp, t.gtab, t.gtabd, t.glo, t.gext, t.ptab, t.pdtab, t.plo);
   }
   const float margin_pt = emd_fp32_d2_margin(g.L, fmax(sp.r_proj, sp.r_loc));
   if (t.te_off)
@@ -912,8 +922,8 @@ void emd_launch_local_force(const GridInfo &g, const SpeciesDev &sp,
                                               : n_atoms <= 9 ? EMD_SPLIT_MAX : 608 / n_atoms;
   dim3 grid(n_atoms, nsplit);
   if (t.gtab)
-    k_local_force_rows<<<grid, 256, 0, st>>>(g.n, g.h, g.L, t.Rw, t.gtab, t.gtabd, sp,
-                                             v_es_a, v_es_b,
+    k_local_force_rows<<<grid, 256, 0, st>>>(g.n, g.h, g.L, t.Rw, t.gtab, t.gtabd,
+                                             t.glo, t.gext, sp, v_es_a, v_es_b,
                                              emd_fp32_d2_margin(g.L, sp.r_loc), part);
   else
     k_local_force<false><<<grid, 256, 0, st>>>(g.n, g.h, g.L, t.Rw, t.gtab, sp,
