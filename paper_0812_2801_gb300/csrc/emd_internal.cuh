@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include "emd.h"
+#include "launch_rules.h"
 
 #define EMD_PT_KMAX 16          // atoms per grid point in the point-major table
 #define EMD_TILE 8              // edge of the tiles that carry atom candidates
@@ -456,7 +457,6 @@ void emd_launch_absdiff_partials(int n3, const double *a, const double *b, doubl
 // X + i n3; complex128 for EMD_FP64, complex64 otherwise): G = scale X^H Y
 // (m x m, column-major FP64, summed in FP64 in a fixed order; part holds
 // emd_gram_scratch(n3, m) double2), and B = X V (V column-major FP64)
-int emd_gram_chunks(int n3, int m);
 size_t emd_gram_scratch(int n3, int m);
 void emd_launch_gram(int prec, const void *X, const void *Y, int n3, int m, double scale,
                      double2 *part, double2 *G, cudaStream_t st);

@@ -109,8 +109,8 @@ __global__ void k_scale_canon(V *c, size_t n3, size_t tot, const double *__restr
 // complex64 read into FP64 sums).  G = h^3 X^H Y, m x m, column-major FP64.
 // k_gram: CTA (row chunk, 16 x 16 tile of G); the chunk's rows pass through
 // shared memory 32 at a time; complex64 products are summed in FP32 over
-// those 32 rows and added to the FP64 sums; the chunks' partial tiles are
-// added in chunk order by k_gram_sum (deterministic).
+// those 32 rows and added to the FP64 sums; k_gram_sum adds the chunks'
+// partial tiles in a fixed order.
 template <typename C> struct GramT;
 template <> struct GramT<double2> {
   __device__ static double2 load(const double2 *p) { return *p; }
@@ -281,13 +281,6 @@ void emd_launch_fill_random(int prec, void *canon, size_t n3, int c0, int c1, un
 
 // G = scale X^H Y (m x m, column-major FP64); part: scratch of
 // emd_gram_scratch(n3, m) double2
-// row chunks of k_gram: enough CTAs for 16 per SM with the (m / 16)^2 tiles of
-// G, of at least 96 rows each.  (n3 / 4096 chunks left 3 CTAs on 24^3 with 9
-// states: 1.23 ms per product, 80 % of the ground state.)
-int emd_gram_chunks(int n3, int m) {
-  const int tiles = ((m + 15) / 16) * ((m + 15) / 16);
-  return std::max(1, std::min((16 * 152 + tiles - 1) / tiles, n3 / 96));
-}
 size_t emd_gram_scratch(int n3, int m) { return (size_t)emd_gram_chunks(n3, m) * m * m; }
 
 void emd_launch_gram(int prec, const void *X, const void *Y, int n3, int m, double scale,
