@@ -13,17 +13,16 @@
 //    are chosen by that cost: few large butterflies (fewest instructions) on
 //    large grids, more small ones (short chains) on small grids;
 //  * the butterflies' own twiddles are constants, prime butterflies use the
-//    real symmetric form (half the multiplications of the direct sum);
+//    real symmetric form (half the multiplications of the direct sum), and
+//    those of coprime factors need no twiddles between them;
 //  * the forward z transform, the spectral factor and the inverse z transform
 //    are one kernel: the spectrum along z never leaves the SM;
-//  * real data run as half-length complex lines (even n) and only kx <= n / 2
-//    is kept.
+//  * two real lines run as one complex line and only kx <= n / 2 is kept.
 // Measured: emd_poisson_static on 48^3 92 -> 54 us a call (seven passes of one
-// exchange per radix 2, 3, 4 or 5 on complex data before); the system's own
-// solve, ncu, cold caches: 48^3 60 -> 55 us, 64^3 94 -> 77 us; on 120^3
-// (54 orbitals, complex64) an MD step with its two solves takes 0.5 ms less.
-// Every pass reads lines that are contiguous and writes 64- or 128-byte pieces
-// of the layout whose next axis is contiguous.
+// exchange per radix 2, 3, 4 or 5 on complex data before); the five kernels
+// alone, 48^3 45 us, 64^3 64 us, 96^3 147 us, 120^3 312 us, 160^3 690 us.
+// Every pass reads lines that are contiguous and writes 64-byte pieces or
+// longer of the layout whose next axis is contiguous.
 //   1 x real -> complex   [z][y][x]   -> [kx][z][y]
 //   2 y                   [kx][z][y]  -> [ky][kx][z]
 //   3 z, factor, inverse z            -> [kx][z][ky]
@@ -31,6 +30,15 @@
 //   5 inverse x, complex -> real      -> [z][y][x]
 // Inverse transforms run the forward butterflies with real and imaginary
 // parts exchanged on the way in and out.
+//
+// Accuracy: a solve is off by about three roundings (2-norm), most of them of
+// the additions: 3.5e-16 on average over 20 grids of 16^3 to 64^3, 3.7e-16 with
+// the complex transforms, 4.2e-16 with lines of n / 2 complex values.  What
+// keeps it there: pairs of real lines average the errors of Z_k and Z_{n-k} (a
+// line as n / 2 complex values adds those of its untangling), coprime
+// butterflies have no twiddles to round, and sqrt(3) / 2 and sqrt(1/2) come with
+// their low parts, since the rounding of a constant that every line meets
+// scales the whole result (27^3: by 2.5e-16).
 #include <atomic>
 #include "emd_internal.cuh"
 
@@ -227,6 +235,17 @@ template <> struct Dft<2> {
     v[1] = csub(a, v[1]);
   }
 };
+// sqrt(3) / 2 to twice the precision
+template <> struct Dft<3> {
+  static __device__ __forceinline__ void run(double2 (&v)[3]) {
+    constexpr double hi = 0.8660254037844386, lo = 5.017542110902451e-17;
+    const double2 t = cadd(v[1], v[2]), d = csub(v[1], v[2]);
+    const double2 a = make_double2(fma(-0.5, t.x, v[0].x), fma(-0.5, t.y, v[0].y));
+    v[0] = cadd(v[0], t);
+    v[1] = make_double2(fma(hi, d.y, fma(lo, d.y, a.x)), fma(-hi, d.x, fma(-lo, d.x, a.y)));
+    v[2] = make_double2(fma(-hi, d.y, fma(-lo, d.y, a.x)), fma(hi, d.x, fma(lo, d.x, a.y)));
+  }
+};
 template <> struct Dft<4> {
   static __device__ __forceinline__ void run(double2 (&v)[4]) {
     const double2 a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
@@ -237,10 +256,17 @@ template <> struct Dft<4> {
     v[3] = make_double2(b.x - d.y, b.y + d.x);
   }
 };
-// v (c - i s) for a constant (c, s); 1, -1, i and -i need no multiplication
+// v (c - i s) for a constant (c, s); 1, -1, i and -i need no multiplication,
+// and the diagonals take sqrt(1/2) to twice the precision
 __device__ __forceinline__ double2 ctwiddle(double2 v, double2 w) {
   if (w.y == 0.0) return w.x > 0.0 ? v : make_double2(-v.x, -v.y);
   if (w.x == 0.0) return w.y > 0.0 ? make_double2(v.y, -v.x) : make_double2(-v.y, v.x);
+  if (w.x == w.y || w.x == -w.y) {
+    constexpr double hi = 0.7071067811865476, lo = -4.833646656726457e-17;
+    const double sx = w.x > 0.0 ? 1.0 : -1.0, sy = w.y > 0.0 ? 1.0 : -1.0;
+    const double a = sx * v.x + sy * v.y, b = sx * v.y - sy * v.x;
+    return make_double2(fma(hi, a, lo * a), fma(hi, b, lo * b));
+  }
   return cmul(v, make_double2(w.x, -w.y));
 }
 // composite R = A B: B transforms of A points, constant twiddles, A of B points
@@ -268,13 +294,42 @@ template <int A, int B> struct DftAB {
     }
   }
 };
-template <> struct Dft<6> : DftAB<2, 3> {};
+// R = A B with A and B coprime: n = (B j + A i) mod R and k = the number that
+// is k_1 mod A and k_2 mod B (Good 1958, Thomas 1963): no twiddles between
+// the B transforms of A points and the A of B points
+template <int A, int B> struct DftCoprime {
+  static __host__ __device__ constexpr int crt(int k1, int k2) {
+    int k = k2;
+    while (k % A != k1) k += B;
+    return k;
+  }
+  static __device__ __forceinline__ void run(double2 (&v)[A * B]) {
+    constexpr int R = A * B;
+    double2 u[B][A];
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+#pragma unroll
+      for (int j = 0; j < A; ++j) u[i][j] = v[(B * j + A * i) % R];
+      Dft<A>::run(u[i]);
+    }
+#pragma unroll
+    for (int k = 0; k < A; ++k) {
+      double2 w[B];
+#pragma unroll
+      for (int i = 0; i < B; ++i) w[i] = u[i][k];
+      Dft<B>::run(w);
+#pragma unroll
+      for (int q = 0; q < B; ++q) v[crt(k, q)] = w[q];
+    }
+  }
+};
+template <> struct Dft<6> : DftCoprime<2, 3> {};
 template <> struct Dft<8> : DftAB<2, 4> {};
 template <> struct Dft<9> : DftAB<3, 3> {};
-template <> struct Dft<10> : DftAB<2, 5> {};
-template <> struct Dft<12> : DftAB<3, 4> {};
-template <> struct Dft<14> : DftAB<2, 7> {};
-template <> struct Dft<15> : DftAB<3, 5> {};
+template <> struct Dft<10> : DftCoprime<2, 5> {};
+template <> struct Dft<12> : DftCoprime<3, 4> {};
+template <> struct Dft<14> : DftCoprime<2, 7> {};
+template <> struct Dft<15> : DftCoprime<3, 5> {};
 template <> struct Dft<16> : DftAB<4, 4> {};
 
 #define EMD_FFT_SWITCH(R, CALL)                                                     \
@@ -297,7 +352,7 @@ template <> struct Dft<16> : DftAB<4, 4> {};
     case 16: CALL(16); break;                                                       \
   }
 
-// A line transform of len = r[0] r[1] .. r[ns-1] points, ns >= 2.  One step
+// A line transform of n = r[0] r[1] .. r[ns-1] points, ns >= 2.  One step
 // turns a block of R m values x[j + m t] into R blocks of m: block k holds
 // w_{Rm}^{jk} sum_t w_R^{tk} x[j + m t] and is the transform of length m that
 // gives the frequencies k, k + R, ...; so a step reads and writes the same
@@ -319,11 +374,10 @@ __device__ __forceinline__ int operator/(int t, const FastDiv &f) {
   return f.d == 1 ? t : (int)__umulhi((unsigned)t, f.mul);
 }
 struct FftLine {
-  int n, len, ns;         // grid edge; line length; steps
+  int n, ns;              // grid edge and line length; steps
   int r[kFftSteps];       // factors
   int m[kFftSteps];       // block length after the step
-  FastDiv by_r[kFftSteps], by_m[kFftSteps], by_blocks;   // by_blocks: len / r[ns - 1]
-  int tw;                 // exp(-2 pi i t / len) = roots[tw t], roots of n
+  FastDiv by_r[kFftSteps], by_m[kFftSteps], by_blocks;   // by_blocks: n / r[ns - 1]
   int lsh;                // 2^lsh lines per CTA
   int ls;                 // shared-memory stride of a line
   int threads;            // per CTA
@@ -358,7 +412,7 @@ __device__ __forceinline__ void first(const FftLine &p, const double2 *rt, doubl
     e[0] = v[0];
 #pragma unroll
     for (int k = 1; k < R; ++k) {
-      w += p.tw * j;                       // root j k
+      w += j;                              // root j k
       e[k * mp] = cmul(v[k], *w);
     }
   }
@@ -379,7 +433,7 @@ __device__ __forceinline__ void middle(const FftLine &p, const double2 *rt, doub
     e[0] = v[0];
 #pragma unroll
     for (int k = 1; k < R; ++k) {
-      w += p.tw * groups * j;
+      w += groups * j;
       e[k * m] = cmul(v[k], *w);
     }
   }
@@ -427,41 +481,26 @@ __device__ __forceinline__ double2 *load_roots(double2 *sm, int n,
   return sm + n;
 }
 
-// 1: x real -> complex.  EVEN: x_2j + i x_2j+1 as a line of n / 2 values,
-// untangled into X_k = E_k + W^k O_k, E_k = (Z_k + conj Z_{m-k}) / 2, O_k =
-// (Z_k - conj Z_{m-k}) / (2i), W = exp(-2 pi i / n), k = 0 .. m.
-template <bool EVEN>
+// 1: x, real -> complex.  Two real lines a, b run as one complex line Z of a +
+// i b; 2 A_k = Z_k + conj Z_{n-k}, 2 i B_k = Z_k - conj Z_{n-k}, k <= n / 2.
 __global__ void __launch_bounds__(256)
-k_fft_x(const double *__restrict__ in, double2 *__restrict__ out, FftLine p,
+k_fft_x(const double *__restrict__ in, double2 *__restrict__ out, FftLine p, int nh,
         const double2 *__restrict__ roots) {
   extern __shared__ double2 sm[];
-  const int n = p.n, nlines = n * n, l0 = blockIdx.x << p.lsh;
+  const int n = p.n, nlines = n * n, l0 = blockIdx.x << (p.lsh + 1);
   double2 *ex = load_roots(sm, n, roots), *zs = ex + (p.ls << p.lsh);
-  if (EVEN) {
-    line_fft<false>(p, sm, ex, [&](int l, int i) {
-      const int line = min(l0 + l, nlines - 1);
-      // two 8-byte loads: a caller's grid may start on any 8-byte boundary
-      const double *x = in + (size_t)line * n + 2 * i;
-      return make_double2(__ldg(x), __ldg(x + 1));
-    }, [&](int l, int k, double2 v) { zs[l * (p.len | 1) + k] = v; });
-    __syncthreads();
-    const int m = p.len;
-    for (int t = threadIdx.x; t < (m + 1) << p.lsh; t += blockDim.x) {
-      const int k = t >> p.lsh, l = t & ((1 << p.lsh) - 1);
-      if (l0 + l >= nlines) continue;
-      const double2 zk = zs[l * (m | 1) + (k == m ? 0 : k)];
-      const double2 zr = zs[l * (m | 1) + (k == 0 ? 0 : m - k)];
-      const double2 e = make_double2(0.5 * (zk.x + zr.x), 0.5 * (zk.y - zr.y));
-      const double2 o = make_double2(0.5 * (zk.y + zr.y), -0.5 * (zk.x - zr.x));
-      out[(size_t)k * nlines + l0 + l] = cadd(e, cmul(sm[k], o));
-    }
-  } else {
-    line_fft<false>(p, sm, ex, [&](int l, int i) {
-      const int line = min(l0 + l, nlines - 1);
-      return make_double2(__ldg(in + (size_t)line * n + i), 0.0);
-    }, [&](int l, int k, double2 v) {
-      if (l0 + l < nlines && 2 * k < n) out[(size_t)k * nlines + l0 + l] = v;
-    });
+  line_fft<false>(p, sm, ex, [&](int l, int i) {
+    // 8-byte loads: a caller's grid may start on any 8-byte boundary
+    const int a = min(l0 + 2 * l, nlines - 1), b = min(a + 1, nlines - 1);
+    return make_double2(__ldg(in + (size_t)a * n + i), __ldg(in + (size_t)b * n + i));
+  }, [&](int l, int k, double2 v) { zs[l * (n | 1) + k] = v; });
+  __syncthreads();
+  for (int t = threadIdx.x; t < nh << p.lsh; t += blockDim.x) {
+    const int k = t >> p.lsh, l = t & ((1 << p.lsh) - 1), a = l0 + 2 * l;
+    const double2 zk = zs[l * (n | 1) + k], zr = zs[l * (n | 1) + (k ? n - k : 0)];
+    double2 *o = out + (size_t)k * nlines + a;
+    if (a < nlines) o[0] = make_double2(zk.x + zr.x, zk.y - zr.y);
+    if (a + 1 < nlines) o[1] = make_double2(zk.y + zr.y, zr.x - zk.x);
   }
 }
 
@@ -528,53 +567,43 @@ k_fft_z_factor(const double2 *__restrict__ in, double2 *__restrict__ out, FftLin
   });
 }
 
-// 5: inverse x.  EVEN: Z_k = (X_k + conj X_{m-k}) + i conj(W^k) (X_k - conj
-// X_{m-k}), k < m, and the inverse half-length transform gives x_2j + i
-// x_2j+1.  Odd n: the full Hermitian line, real parts kept.
-template <bool EVEN>
+// 5: inverse x, two Hermitian lines A, B as one: Z_k = A_k + i B_k, Z_{n-k} =
+// conj A_k + i conj B_k; the imaginary parts that rounding left at k = 0 and n
+// / 2 are dropped.
 __global__ void __launch_bounds__(256)
 k_fft_x_inv(const double2 *__restrict__ in, double *__restrict__ out, FftLine p, int nh,
             const double2 *__restrict__ roots) {
   extern __shared__ double2 sm[];
-  const int n = p.n, nlines = n * n, l0 = blockIdx.x << p.lsh;
-  double2 *ex = load_roots(sm, n, roots), *xs = ex + (p.ls << p.lsh);
+  const int n = p.n, nlines = n * n, l0 = blockIdx.x << (p.lsh + 1);
+  double2 *ex = load_roots(sm, n, roots), *zs = ex + (p.ls << p.lsh);
   for (int t = threadIdx.x; t < nh << p.lsh; t += blockDim.x) {
-    const int l = t / nh, k = t - l * nh, line = min(l0 + l, nlines - 1);
-    xs[l * nh + k] = __ldg(in + (size_t)line * nh + k);
+    const int l = t / nh, k = t - l * nh;
+    const int la = min(l0 + 2 * l, nlines - 1), lb = min(la + 1, nlines - 1);
+    const double2 a = __ldg(in + (size_t)la * nh + k), b = __ldg(in + (size_t)lb * nh + k);
+    double2 *z = zs + l * (n | 1);
+    if (k == 0 || 2 * k == n) {
+      z[k] = make_double2(b.x, a.x);                          // exchanged: inverse
+    } else {
+      z[k] = make_double2(a.y + b.x, a.x - b.y);
+      z[n - k] = make_double2(b.x - a.y, a.x + b.y);
+    }
   }
   __syncthreads();
-  if (EVEN) {
-    const int m = p.len;
-    line_fft<true>(p, sm, ex, [&](int l, int k) {
-      const double2 xk = xs[l * nh + k], xr = xs[l * nh + m - k];
-      const double2 sp = make_double2(xk.x + xr.x, xk.y - xr.y);
-      const double2 df = make_double2(xk.x - xr.x, xk.y + xr.y);
-      const double2 w = sm[k];
-      const double2 t = cmul(make_double2(w.x, -w.y), df);
-      return make_double2(sp.y + t.x, sp.x - t.y);             // exchanged: inverse
-    }, [&](int l, int k, double2 v) {
-      if (l0 + l >= nlines) return;
-      double *x = out + (size_t)(l0 + l) * n + 2 * k;
-      x[0] = v.y;
-      x[1] = v.x;
-    });
-  } else {
-    line_fft<true>(p, sm, ex, [&](int l, int k) {
-      const double2 v = xs[l * nh + (k < nh ? k : n - k)];
-      return make_double2(k < nh ? v.y : -v.y, v.x);           // exchanged: inverse
-    }, [&](int l, int k, double2 v) {
-      if (l0 + l < nlines) out[(size_t)(l0 + l) * n + k] = v.y;
-    });
-  }
+  line_fft<true>(p, sm, ex, [&](int l, int k) { return zs[l * (n | 1) + k]; },
+                 [&](int l, int k, double2 v) {
+    const int a = l0 + 2 * l;
+    if (a < nlines) out[(size_t)a * n + k] = v.y;
+    if (a + 1 < nlines) out[(size_t)(a + 1) * n + k] = v.x;
+  });
 }
 
-// FP64 instructions of a butterfly and its R - 1 twiddle products
+// about the FP64 instructions of a butterfly, and its R - 1 twiddle products
 int butterfly_cost(int R) {
   static const int dft[17] = {0, 0, 4, 14, 16, 36, 44, 66, 64, 100, 92, 150, 108, 210, 156, 170, 160};
   return dft[R] + 4 * (R - 1);
 }
 
-// the cheapest way to write len as 2 to 4 factors of at most 16, in ascending
+// the cheapest way to write n as 2 to 4 factors of at most 16, in ascending
 // order: a step costs its instructions times 64 cycles times the warps per
 // scheduler (at least one), and about 1500 cycles for its exchange
 void best_factors(FftLine &p, int nlines, int ns, int at, int left, int lo, int *r, double c,
@@ -582,7 +611,7 @@ void best_factors(FftLine &p, int nlines, int ns, int at, int left, int lo, int 
   if (at == ns - 1) {
     if (left > 16 || left < lo) return;
     r[at] = left;
-    const double w = (double)nlines * (p.len / left) / 32.0 / 608.0;
+    const double w = (double)nlines * (p.n / left) / 32.0 / 608.0;
     c += (w > 1.0 ? w : 1.0) * (butterfly_cost(left) - 4 * (left - 1)) * 64.0;
     if (c >= best) return;
     best = c;
@@ -592,43 +621,42 @@ void best_factors(FftLine &p, int nlines, int ns, int at, int left, int lo, int 
   }
   for (int f = lo; f <= 16; ++f) {
     if (left % f) continue;
-    const double w = (double)nlines * (p.len / f) / 32.0 / 608.0;
+    const double w = (double)nlines * (p.n / f) / 32.0 / 608.0;
     r[at] = f;
     best_factors(p, nlines, ns, at + 1, left / f, f, r,
                  c + 1500.0 + (w > 1.0 ? w : 1.0) * butterfly_cost(f) * 64.0, best);
   }
 }
 
-// false: len is not a product of four factors of at most 16
-bool line_plan(FftLine &p, int n, int len, int nlines) {
+// false: n is not a product of four factors of at most 16
+bool line_plan(FftLine &p, int n) {
+  const int nlines = n * (n / 2 + 1);
   p.n = n;
-  p.len = len;
   p.ns = 0;
   int r[kFftSteps];
   double best = 1e300;
-  for (int ns = 2; ns <= kFftSteps; ++ns) best_factors(p, nlines, ns, 0, len, 1, r, 0.0, best);
+  for (int ns = 2; ns <= kFftSteps; ++ns) best_factors(p, nlines, ns, 0, n, 1, r, 0.0, best);
   if (!p.ns) return false;
-  int m = len;
+  int m = n;
   for (int s = 0; s < p.ns; ++s) {
     p.m[s] = m /= p.r[s];
     p.by_r[s] = fast_div(p.r[s]);
     p.by_m[s] = fast_div(p.m[s]);
   }
-  p.by_blocks = fast_div(len / p.r[p.ns - 1]);
-  p.tw = n / len;
+  p.by_blocks = fast_div(n / p.r[p.ns - 1]);
   p.ls = (p.r[0] * (p.m[0] | 1)) | 1;
   // 8 lines: transposed writes of 128 bytes; 4 where two copies of the lines
   // and the roots pass 200 KB
   p.lsh = (8 * (p.ls + n + 1) + n) * (int)sizeof(double2) <= 200 * 1024 ? 3 : 2;
-  const int most = (len / p.r[0]) << p.lsh;            // threads of the widest step
+  const int most = (n / p.r[0]) << p.lsh;              // threads of the widest step
   p.threads = most >= 256 ? 256 : (most + 31) / 32 * 32;
   return true;
 }
 
-// The two line plans of a grid (x, and y or z), worked out once per size and
-// kept for the life of the process.
+// The line plan of a grid, worked out once per size and kept for the life of
+// the process.
 struct FftPlan {
-  FftLine x, y;
+  FftLine line;
   bool ok;
 };
 constexpr int kFftMaxN = 1024;
@@ -638,8 +666,7 @@ const FftPlan *plan_of(int n) {
   const FftPlan *p = kept[n].load();
   if (!p) {
     FftPlan *q = new FftPlan();
-    const int nh = n / 2 + 1;                     // (n + 1) / 2 for odd n
-    q->ok = line_plan(q->x, n, n % 2 ? n : n / 2, n * n) && line_plan(q->y, n, n, nh * n);
+    q->ok = line_plan(q->line, n);
     if (kept[n].compare_exchange_strong(p, q)) p = q;
     else delete q;
   }
@@ -650,13 +677,11 @@ const FftPlan *plan_of(int n) {
 // roots, 144 KB (once per process and device; setting it again changes nothing)
 void allow_large_shared() {
   const int most = 200 * 1024;
-  cudaFuncSetAttribute(k_fft_x<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  cudaFuncSetAttribute(k_fft_x<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(k_fft_x, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   cudaFuncSetAttribute(k_fft_y<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   cudaFuncSetAttribute(k_fft_y<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   cudaFuncSetAttribute(k_fft_z_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  cudaFuncSetAttribute(k_fft_x_inv<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  cudaFuncSetAttribute(k_fft_x_inv<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(k_fft_x_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
 }  // namespace
@@ -669,23 +694,18 @@ bool emd_fft2_ok(int n) { return plan_of(n) != nullptr; }
 void emd_fft2_multiply(int n, const double *in, double *out, double2 *wa, double2 *wb,
                        const double2 *roots, double c, double kappa, const double *inv_s,
                        cudaStream_t st) {
-  const bool even = n % 2 == 0;
   const int nh = n / 2 + 1;                       // (n + 1) / 2 for odd n
-  const FftLine &px = plan_of(n)->x, &py = plan_of(n)->y;
-  const int lx = 1 << px.lsh, ly = 1 << py.lsh;
-  const int bx = (n * n + lx - 1) / lx, by = (nh * n + ly - 1) / ly;
+  const FftLine &p = plan_of(n)->line;
+  const int per = 1 << p.lsh;
+  const int bx = (n * n + 2 * per - 1) / (2 * per), by = (nh * n + per - 1) / per;
   const size_t c16 = sizeof(double2);
-  const size_t sx = (n + (size_t)lx * (px.ls + (px.len | 1))) * c16;
-  const size_t sxi = (n + (size_t)lx * (px.ls + nh)) * c16;
-  const size_t sy = (n + (size_t)ly * py.ls) * c16;
-  const size_t sz = (n + (size_t)ly * (py.ls + (n | 1))) * c16;
-  if (sz > 49152) allow_large_shared();
+  const size_t one = (n + (size_t)per * p.ls) * c16, two = one + (size_t)per * (n | 1) * c16;
+  if (two > 49152) allow_large_shared();
   const FastDiv by_n = fast_div(n), by_nh = fast_div(nh);
-  if (even) k_fft_x<true><<<bx, px.threads, sx, st>>>(in, wa, px, roots);
-  else k_fft_x<false><<<bx, px.threads, sx, st>>>(in, wa, px, roots);
-  k_fft_y<false><<<by, py.threads, sy, st>>>(wa, wb, py, nh, by_nh, roots);
-  k_fft_z_factor<<<by, py.threads, sz, st>>>(wb, wa, py, nh, by_n, c, kappa, inv_s, roots);
-  k_fft_y<true><<<by, py.threads, sy, st>>>(wa, wb, py, nh, by_nh, roots);
-  if (even) k_fft_x_inv<true><<<bx, px.threads, sxi, st>>>(wb, out, px, nh, roots);
-  else k_fft_x_inv<false><<<bx, px.threads, sxi, st>>>(wb, out, px, nh, roots);
+  k_fft_x<<<bx, p.threads, two, st>>>(in, wa, p, nh, roots);
+  k_fft_y<false><<<by, p.threads, one, st>>>(wa, wb, p, nh, by_nh, roots);
+  // pass 1 leaves twice the spectrum
+  k_fft_z_factor<<<by, p.threads, two, st>>>(wb, wa, p, nh, by_n, 0.5 * c, kappa, inv_s, roots);
+  k_fft_y<true><<<by, p.threads, one, st>>>(wa, wb, p, nh, by_nh, roots);
+  k_fft_x_inv<<<bx, p.threads, two, st>>>(wb, out, p, nh, roots);
 }

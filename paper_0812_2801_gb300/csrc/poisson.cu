@@ -178,10 +178,15 @@ void spectral_multiply(const GridInfo &g, const double *charge, double *v, doubl
 
 }  // namespace
 
+// 4 pi / ((2 pi / L)^2 N^3) with L = n h, rounded once
+static double poisson_scale(int n, double h) {
+  const long double PI_L = 3.141592653589793238462643383279502884L;
+  return (double)((long double)h * h / (PI_L * n));
+}
+
 void emd_launch_poisson(const GridInfo &g, const double *charge, double *v,
                         double2 *wa, double2 *wb, cudaStream_t st) {
-  const double gq = 2.0 * M_PI / g.L;
-  spectral_multiply(g, charge, v, wa, wb, 4.0 * M_PI / (gq * gq) / (double)g.n3, -1.0, st);
+  spectral_multiply(g, charge, v, wa, wb, poisson_scale(g.n, g.h), -1.0, st);
 }
 
 void emd_launch_kerker(const GridInfo &g, double q0, const double *r, double *out,
@@ -264,13 +269,19 @@ cudaError_t static_scratch(double2 **out) {
   return cudaSuccess;
 }
 
-// roots: exp(-2 pi i t / n), t < n; inv_s[s] = 1 / s, s = 1 .. smax, 0 at 0
+// roots: exp(-2 pi i t / n), t < n; inv_s[s] = 1 / s, s = 1 .. smax, 0 at 0.
+// An angle is brought to its octant in integers first: the rounding of -2 t /
+// n as an argument near 2 would turn the root by up to 3.5e-16.
 __global__ void k_fill_tables(int n, double2 *roots, int smax, double *inv_s) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n) {
-    double sn, cs;
-    sincospi(-2.0 * (double)t / (double)n, &sn, &cs);
-    roots[t] = make_double2(cs, sn);
+    const int o = 8 * t / n;                                  // octant
+    const int num = o & 1 ? (o + 1) * n - 8 * t : 8 * t - o * n;
+    double sn, cs;                                            // 0 .. pi / 4
+    sincospi((double)num / (double)(4 * n), &sn, &cs);
+    const bool swap = (o + 1) & 2;                            // octants 1, 2, 5, 6
+    const double x = swap ? sn : cs, y = swap ? cs : sn;
+    roots[t] = make_double2(o >= 2 && o < 6 ? -x : x, o < 4 ? -y : y);
   }
   if (t <= smax) inv_s[t] = t ? 1.0 / (double)t : 0.0;
 }
@@ -290,15 +301,12 @@ extern "C" int emd_poisson_static(int n, double h, const double *charge,
   if (static_scratch(&base) != cudaSuccess)
     return emd_set_error(EMD_ECUDA, "emd_poisson_static: cudaGetSymbolAddress of "
                                     "the static scratch failed");
-  const size_t n3 = (size_t)n * n * n;
   double2 *wa = base, *wb = base + kStaticN3, *tab = base + 2 * kStaticN3;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  const double gq = 2.0 * M_PI / (n * h);
   double *inv_s = reinterpret_cast<double *>(tab + kStaticMaxN);
   const int smax = 3 * (n / 2) * (n / 2);
   k_fill_tables<<<smax / 64 + 1, 64, 0, st>>>(n, tab, smax, inv_s);
-  emd_fft2_multiply(n, charge, v, wa, wb, tab, 4.0 * M_PI / (gq * gq) / (double)n3, -1.0, inv_s,
-                    st);
+  emd_fft2_multiply(n, charge, v, wa, wb, tab, poisson_scale(n, h), -1.0, inv_s, st);
   if (cudaGetLastError() != cudaSuccess)
     return emd_set_error(EMD_ECUDA, "emd_poisson_static: kernel launch failed");
   return emd_set_error(EMD_OK, "");
