@@ -405,7 +405,7 @@ void emd_launch_vv_velocities(int n_atoms, const double *F_loc,
                               double *V, double dt, double mass, int update_v,
                               cudaStream_t st);
 
-// fft2.cu: spectral multiplication in five kernels
+// fft2.cu: spectral multiplication in five launches
 bool emd_fft2_ok(int n);
 void emd_fft2_multiply(int n, const double *in, double *out, double2 *wa, double2 *wb,
                        const double2 *roots, double c, double kappa, const double *inv_s,

@@ -1,4 +1,4 @@
-// Spectral multiplication on periodic grids in five kernels: the transforms of
+// Spectral multiplication on periodic grids in five passes: the transforms of
 // the Hartree and ionic electrostatics (eq. E_KS, eq. ionicpotential; a
 // periodic spectral solve stands in for the paper's finite-system solver) and
 // of Kerker's preconditioner.
@@ -16,18 +16,18 @@
 //    real symmetric form (half the multiplications of the direct sum), and
 //    those of coprime factors need no twiddles between them;
 //  * the forward z transform, the spectral factor and the inverse z transform
-//    are one kernel: the spectrum along z never leaves the SM;
+//    are one pass: the spectrum along z never leaves the SM;
 //  * two real lines run as one complex line and only kx <= n / 2 is kept.
-// Measured: emd_poisson_static on 48^3 92 -> 54 us a call (seven passes of one
-// exchange per radix 2, 3, 4 or 5 on complex data before); the five kernels
-// alone, 48^3 45 us, 64^3 64 us, 96^3 147 us, 120^3 312 us, 160^3 690 us.
+// Measured: emd_poisson_static on 48^3 92 -> 51 us a call (seven passes of one
+// exchange per radix 2, 3, 4 or 5 on complex data before); the five passes
+// alone, 48^3 45 us, 64^3 63 us, 96^3 148 us, 120^3 311 us, 160^3 687 us.
 // Every pass reads lines that are contiguous and writes 64-byte pieces or
 // longer of the layout whose next axis is contiguous.
-//   1 x real -> complex   [z][y][x]   -> [kx][z][y]
-//   2 y                   [kx][z][y]  -> [ky][kx][z]
-//   3 z, factor, inverse z            -> [kx][z][ky]
-//   4 inverse y                       -> [z][y][kx]
-//   5 inverse x, complex -> real      -> [z][y][x]
+//   X    x, real -> complex       [z][y][x]    -> [kx][z][y]
+//   Y    y                        [kx][z][y]   -> [ky][kx][z]
+//   Z    z, factor, inverse z     [ky][kx][z]  -> [kx][z][ky]
+//   YINV inverse y                [kx][z][ky]  -> [z][y][kx]
+//   XINV inverse x, complex -> real [z][y][kx] -> [z][y][x]
 // Inverse transforms run the forward butterflies with real and imaginary
 // parts exchanged on the way in and out.
 //
@@ -377,6 +377,7 @@ struct FftLine {
   int n, ns;              // grid edge and line length; steps
   int r[kFftSteps];       // factors
   int m[kFftSteps];       // block length after the step
+  FastDiv by_n, by_nh;    // nh: n / 2 + 1
   FastDiv by_r[kFftSteps], by_m[kFftSteps], by_blocks;   // by_blocks: n / r[ns - 1]
   int lsh;                // 2^lsh lines per CTA
   int ls;                 // shared-memory stride of a line
@@ -396,205 +397,225 @@ __device__ __forceinline__ int block_at(const FftLine &p, int kk, int steps) {
   return off + q * p.m[steps - 1];
 }
 
-// The roots are read from shared memory (rt, copied at the kernel's start).
-// first step: ld(l, i) gives element i of line l
-template <int R, typename LD>
-__device__ __forceinline__ void first(const FftLine &p, const double2 *rt, double2 *ex, LD ld) {
-  const int m = p.m[0], mp = m | 1;
-  for (int t = threadIdx.x; t < m << p.lsh; t += blockDim.x) {
-    const int l = t / p.by_m[0], j = t - l * m;
-    double2 v[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = ld(l, j + r * m);
-    Dft<R>::run(v);
-    double2 *e = ex + l * p.ls + j;
-    const double2 *w = rt;
-    e[0] = v[0];
-#pragma unroll
-    for (int k = 1; k < R; ++k) {
-      w += j;                              // root j k
-      e[k * mp] = cmul(v[k], *w);
+// The five passes are one kernel: the butterflies of 1 to 16 points are nearly
+// all of its code, and the first solve of a process waits until the code is on
+// the GPU (48^3: 0.7 ms for 0.5 MB; five kernels with a copy per transform were
+// 4 MB and took 14 ms).
+//   X    real -> complex.  Two real lines a, b run as one complex line Z of a
+//        + i b; 2 A_k = Z_k + conj Z_{n-k}, 2 i B_k = Z_k - conj Z_{n-k}, k <=
+//        n / 2: twice the spectrum.
+//   Y    lines (kx, z) along y
+//   Z    lines (kx, ky) along z: forward, times the factor of the integer s =
+//        mx^2 + my^2 + mz^2 (|G|^2 = (2 pi / L)^2 s), inverse.  kappa < 0: the
+//        Poisson kernel c / s, 0 at s = 0 (inv_s[s] = 1 / s, inv_s[0] = 0);
+//        else Kerker's c s / (s + kappa), c at s = 0.
+//   YINV lines (z, kx) along ky
+//   XINV two Hermitian lines A, B as one: Z_k = A_k + i B_k, Z_{n-k} = conj A_k
+//        + i conj B_k; the imaginary parts that rounding left at k = 0 and n /
+//        2 are dropped.
+enum FftPass { FFT_X, FFT_Y, FFT_Z, FFT_YINV, FFT_XINV };
+
+// Shared memory of a CTA: the plan | roots | exchange array | lines in natural
+// order (line l, element i at l (n | 1) + i).
+struct FftCta {
+  FftPass pass;
+  int l0, nlines;               // first line; lines of the pass
+  const double2 *in;
+  double2 *out;
+  const FftLine *p;
+  double2 *roots, *ex, *nat;
+  bool from_nat, to_nat, swap_in, swap_out;    // this transform's ends
+  // where line l of the CTA starts; its elements are contiguous
+  __device__ __forceinline__ const double2 *source(int l) const {
+    const int n = p->n, nh = (int)p->by_nh.d;
+    if (from_nat) return nat + l * (n | 1);
+    int line = min(l0 + l, nlines - 1);
+    if (pass == FFT_Z) {
+      const int kx = line / p->by_n;
+      line = (line - kx * n) * nh + kx;
+    } else if (pass == FFT_YINV) {
+      const int z = line / p->by_nh;
+      line = (line - z * nh) * n + z;
     }
+    return in + (size_t)line * n;
   }
-}
-// step s in the middle; groups = product of the factors before it
-template <int R>
-__device__ __forceinline__ void middle(const FftLine &p, const double2 *rt, double2 *ex, int s,
-                                       int groups) {
-  const int m = p.m[s];
+  // where its frequency 0 goes (nullptr: no such line), and the step to the next
+  __device__ __forceinline__ double2 *target(int l, size_t &step) const {
+    const int n = p->n, nh = (int)p->by_nh.d, line = l0 + l;
+    step = 1;
+    if (to_nat) return nat + l * (n | 1);
+    if (line >= nlines) return nullptr;
+    if (pass == FFT_Y) {
+      step = nlines;
+      return out + line;
+    }
+    if (pass == FFT_Z) {
+      const int kx = line / p->by_n, ky = line - kx * n;
+      step = n;
+      return out + (size_t)kx * n * n + ky;
+    }
+    const int z = line / p->by_nh, kx = line - z * nh;
+    step = nh;
+    return out + (size_t)z * n * nh + kx;
+  }
+};
+
+// step s but the last, into the exchange array; groups = product of the
+// factors before it.  The first reads the lines' source, the others what
+// they overwrite.
+template <int R> __device__ __forceinline__ void step(const FftCta &f, int s, int groups) {
+  const FftLine &p = *f.p;
+  const int m = p.m[s], st = s ? m : m | 1;
   for (int t = threadIdx.x; t < (groups * m) << p.lsh; t += blockDim.x) {
     const int b = t / p.by_m[s], j = t - b * m, l = b & ((1 << p.lsh) - 1), g = b >> p.lsh;
-    double2 *e = ex + l * p.ls + block_at(p, g, s) + j;
+    double2 *e = f.ex + l * p.ls + (s ? block_at(p, g, s) : 0) + j;
+    const double2 *x = s ? e : f.source(l) + j;
     double2 v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = e[r * m];
+    for (int r = 0; r < R; ++r) v[r] = x[r * m];
+    if (!s && f.swap_in) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = cswap(v[r]);
+    }
     Dft<R>::run(v);
-    const double2 *w = rt;
+    const double2 *w = f.roots;
     e[0] = v[0];
 #pragma unroll
     for (int k = 1; k < R; ++k) {
-      w += groups * j;
-      e[k * m] = cmul(v[k], *w);
+      w += groups * j;                     // root j k groups
+      e[k * st] = cmul(v[k], *w);
     }
   }
 }
-// last step: st(l, k, X_k).  ALONG: neighbouring threads take neighbouring
-// frequencies of a line instead of neighbouring lines.
-template <int R, bool ALONG, typename ST>
-__device__ __forceinline__ void last(const FftLine &p, const double2 *ex, ST st) {
+// the last step, to the lines' target; neighbouring threads take neighbouring lines
+template <int R> __device__ __forceinline__ void last(const FftCta &f) {
+  const FftLine &p = *f.p;
   const int per = (int)p.by_blocks.d;
   for (int t = threadIdx.x; t < per << p.lsh; t += blockDim.x) {
-    const int l = ALONG ? t / p.by_blocks : t & ((1 << p.lsh) - 1);
-    const int k = ALONG ? t - l * per : t >> p.lsh;
-    const double2 *e = ex + l * p.ls + block_at(p, k, p.ns - 1);
+    const int l = t & ((1 << p.lsh) - 1), k = t >> p.lsh;
+    const double2 *e = f.ex + l * p.ls + block_at(p, k, p.ns - 1);
     double2 v[R];
 #pragma unroll
     for (int j = 0; j < R; ++j) v[j] = e[j];
     Dft<R>::run(v);
+    size_t next;
+    double2 *o = f.target(l, next);
+    if (!o) continue;
+    o += k * next;
+    next *= per;
+    if (f.swap_out) {
 #pragma unroll
-    for (int q = 0; q < R; ++q) st(l, k + per * q, v[q]);
+      for (int q = 0; q < R; ++q) v[q] = cswap(v[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < R; ++q) o[q * next] = v[q];
   }
 }
 
-template <bool ALONG, typename LD, typename ST>
-__device__ __forceinline__ void line_fft(const FftLine &p, const double2 *rt, double2 *ex, LD ld,
-                                         ST st) {
-#define EMD_FIRST(R) first<R>(p, rt, ex, ld)
-  EMD_FFT_SWITCH(p.r[0], EMD_FIRST)
-  int groups = p.r[0];
-  for (int s = 1; s < p.ns - 1; ++s) {
-    __syncthreads();
-#define EMD_MIDDLE(R) middle<R>(p, rt, ex, s, groups)
-    EMD_FFT_SWITCH(p.r[s], EMD_MIDDLE)
+__device__ __forceinline__ void line_fft(const FftCta &f) {
+  const FftLine &p = *f.p;
+  int groups = 1;
+  for (int s = 0; s < p.ns - 1; ++s) {
+#define EMD_STEP(R) step<R>(f, s, groups)
+    EMD_FFT_SWITCH(p.r[s], EMD_STEP)
     groups *= p.r[s];
+    __syncthreads();
   }
-  __syncthreads();
-#define EMD_LAST(R) last<R, ALONG>(p, ex, st)
+#define EMD_LAST(R) last<R>(f)
   EMD_FFT_SWITCH(p.r[p.ns - 1], EMD_LAST)
 }
 
-// shared memory: roots | exchange array | second copy of the lines
-__device__ __forceinline__ double2 *load_roots(double2 *sm, int n,
-                                               const double2 *__restrict__ roots) {
-  for (int t = threadIdx.x; t < n; t += blockDim.x) sm[t] = __ldg(roots + t);
-  __syncthreads();
-  return sm + n;
-}
-
-// 1: x, real -> complex.  Two real lines a, b run as one complex line Z of a +
-// i b; 2 A_k = Z_k + conj Z_{n-k}, 2 i B_k = Z_k - conj Z_{n-k}, k <= n / 2.
 __global__ void __launch_bounds__(256)
-k_fft_x(const double *__restrict__ in, double2 *__restrict__ out, FftLine p, int nh,
-        const double2 *__restrict__ roots) {
-  extern __shared__ double2 sm[];
-  const int n = p.n, nlines = n * n, l0 = blockIdx.x << (p.lsh + 1);
-  double2 *ex = load_roots(sm, n, roots), *zs = ex + (p.ls << p.lsh);
-  line_fft<false>(p, sm, ex, [&](int l, int i) {
-    // 8-byte loads: a caller's grid may start on any 8-byte boundary
-    const int a = min(l0 + 2 * l, nlines - 1), b = min(a + 1, nlines - 1);
-    return make_double2(__ldg(in + (size_t)a * n + i), __ldg(in + (size_t)b * n + i));
-  }, [&](int l, int k, double2 v) { zs[l * (n | 1) + k] = v; });
-  __syncthreads();
-  for (int t = threadIdx.x; t < nh << p.lsh; t += blockDim.x) {
-    const int k = t >> p.lsh, l = t & ((1 << p.lsh) - 1), a = l0 + 2 * l;
-    const double2 zk = zs[l * (n | 1) + k], zr = zs[l * (n | 1) + (k ? n - k : 0)];
-    double2 *o = out + (size_t)k * nlines + a;
-    if (a < nlines) o[0] = make_double2(zk.x + zr.x, zk.y - zr.y);
-    if (a + 1 < nlines) o[1] = make_double2(zk.y + zr.y, zr.x - zk.x);
-  }
-}
-
-// 2: lines (kx, z) along y, [kx][z][y] -> [ky][kx][z].  4 (INV): lines (z, kx)
-// along ky, [kx][z][ky] -> [z][y][kx].
-template <bool INV>
-__global__ void __launch_bounds__(256)
-k_fft_y(const double2 *__restrict__ in, double2 *__restrict__ out, FftLine p, int nh, FastDiv by_nh,
-        const double2 *__restrict__ roots) {
-  extern __shared__ double2 sm[];
-  const int n = p.n, nlines = nh * n, l0 = blockIdx.x << p.lsh;
-  double2 *ex = load_roots(sm, n, roots);
-  line_fft<false>(p, sm, ex, [&](int l, int i) {
-    const int line = min(l0 + l, nlines - 1);
-    if (!INV) return __ldg(in + (size_t)line * n + i);
-    const int z = line / by_nh, kx = line - z * nh;
-    return cswap(__ldg(in + ((size_t)kx * n + z) * n + i));
-  }, [&](int l, int k, double2 v) {
-    const int line = l0 + l;
-    if (line >= nlines) return;
-    if (!INV) {
-      out[(size_t)k * nlines + line] = v;
-    } else {
-      const int z = line / by_nh, kx = line - z * nh;
-      out[((size_t)z * n + k) * nh + kx] = cswap(v);
+k_fft(FftPass pass, const void *__restrict__ vin, void *__restrict__ vout,
+      const __grid_constant__ FftLine p, double c, double kappa,
+      const double *__restrict__ inv_s, const double2 *__restrict__ roots) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  const int n = p.n, nh = n / 2 + 1, stride = n | 1;
+  const bool real = pass == FFT_X || pass == FFT_XINV;       // two lines as one
+  FftCta f;
+  f.pass = pass;
+  f.nlines = n * (real ? n : nh);
+  f.l0 = blockIdx.x << (p.lsh + real);
+  f.in = static_cast<const double2 *>(vin);
+  f.out = static_cast<double2 *>(vout);
+  f.p = &p;
+  f.roots = reinterpret_cast<double2 *>(sm);
+  f.ex = f.roots + n;
+  f.nat = f.ex + (p.ls << p.lsh);
+  f.from_nat = real;
+  f.to_nat = real || pass == FFT_Z;
+  f.swap_in = pass == FFT_YINV;
+  f.swap_out = pass == FFT_YINV;
+  for (int t = threadIdx.x; t < n; t += blockDim.x) f.roots[t] = __ldg(roots + t);
+  if (pass == FFT_X) {
+    const double *x = static_cast<const double *>(vin);
+#pragma unroll 4
+    for (int t = threadIdx.x; t < n << p.lsh; t += blockDim.x) {
+      const int l = t / p.by_n, i = t - l * n;
+      // 8-byte loads: a caller's grid may start on any 8-byte boundary
+      const int a = min(f.l0 + 2 * l, f.nlines - 1), b = min(a + 1, f.nlines - 1);
+      f.nat[l * stride + i] =
+          make_double2(__ldg(x + (size_t)a * n + i), __ldg(x + (size_t)b * n + i));
     }
-  });
-}
-
-// 3: lines (kx, ky) along z: forward, times the factor of the integer s = mx^2
-// + my^2 + mz^2 (|G|^2 = (2 pi / L)^2 s), inverse.  kappa < 0: the Poisson
-// kernel c / s, 0 at s = 0 (inv_s[s] = 1 / s, inv_s[0] = 0); else Kerker's c s / (s
-// + kappa), c at s = 0.  [ky][kx][z] -> [kx][z][ky].
-__global__ void __launch_bounds__(256)
-k_fft_z_factor(const double2 *__restrict__ in, double2 *__restrict__ out, FftLine p, int nh, FastDiv by_n,
-               double c, double kappa, const double *__restrict__ inv_s,
-               const double2 *__restrict__ roots) {
-  extern __shared__ double2 sm[];
-  const int n = p.n, nlines = nh * n, l0 = blockIdx.x << p.lsh;
-  double2 *ex = load_roots(sm, n, roots), *zs = ex + (p.ls << p.lsh);
-  line_fft<false>(p, sm, ex, [&](int l, int i) {
-    const int line = min(l0 + l, nlines - 1);
-    const int kx = line / by_n, ky = line - kx * n;
-    return __ldg(in + ((size_t)ky * nh + kx) * n + i);
-  }, [&](int l, int k, double2 v) {
-    const int line = min(l0 + l, nlines - 1);
-    const int kx = line / by_n, ky = line - kx * n;
-    const int my = 2 * ky < n ? ky : ky - n, mz = 2 * k < n ? k : k - n;
-    const int s = kx * kx + my * my + mz * mz;
-    double f;
-    if (kappa < 0.0)
-      f = c * __ldg(inv_s + s);
-    else
-      f = s == 0 ? c : c * (double)s / ((double)s + kappa);
-    zs[l * (n | 1) + k] = make_double2(f * v.y, f * v.x);      // exchanged: inverse
-  });
-  __syncthreads();
-  line_fft<false>(p, sm, ex, [&](int l, int i) { return zs[l * (n | 1) + i]; },
-                  [&](int l, int z, double2 v) {
-    const int line = l0 + l;
-    if (line >= nlines) return;
-    const int kx = line / by_n, ky = line - kx * n;
-    out[((size_t)kx * n + z) * n + ky] = cswap(v);
-  });
-}
-
-// 5: inverse x, two Hermitian lines A, B as one: Z_k = A_k + i B_k, Z_{n-k} =
-// conj A_k + i conj B_k; the imaginary parts that rounding left at k = 0 and n
-// / 2 are dropped.
-__global__ void __launch_bounds__(256)
-k_fft_x_inv(const double2 *__restrict__ in, double *__restrict__ out, FftLine p, int nh,
-            const double2 *__restrict__ roots) {
-  extern __shared__ double2 sm[];
-  const int n = p.n, nlines = n * n, l0 = blockIdx.x << (p.lsh + 1);
-  double2 *ex = load_roots(sm, n, roots), *zs = ex + (p.ls << p.lsh);
-  for (int t = threadIdx.x; t < nh << p.lsh; t += blockDim.x) {
-    const int l = t / nh, k = t - l * nh;
-    const int la = min(l0 + 2 * l, nlines - 1), lb = min(la + 1, nlines - 1);
-    const double2 a = __ldg(in + (size_t)la * nh + k), b = __ldg(in + (size_t)lb * nh + k);
-    double2 *z = zs + l * (n | 1);
-    if (k == 0 || 2 * k == n) {
-      z[k] = make_double2(b.x, a.x);                          // exchanged: inverse
-    } else {
-      z[k] = make_double2(a.y + b.x, a.x - b.y);
-      z[n - k] = make_double2(b.x - a.y, a.x + b.y);
+  } else if (pass == FFT_XINV) {
+#pragma unroll 4
+    for (int t = threadIdx.x; t < nh << p.lsh; t += blockDim.x) {
+      const int l = t / p.by_nh, k = t - l * nh;
+      const int la = min(f.l0 + 2 * l, f.nlines - 1), lb = min(la + 1, f.nlines - 1);
+      const double2 a = __ldg(f.in + (size_t)la * nh + k), b = __ldg(f.in + (size_t)lb * nh + k);
+      double2 *z = f.nat + l * stride;
+      // exchanged: inverse
+      if (k == 0 || 2 * k == n) {
+        z[k] = make_double2(b.x, a.x);
+      } else {
+        z[k] = make_double2(a.y + b.x, a.x - b.y);
+        z[n - k] = make_double2(b.x - a.y, a.x + b.y);
+      }
     }
   }
   __syncthreads();
-  line_fft<true>(p, sm, ex, [&](int l, int k) { return zs[l * (n | 1) + k]; },
-                 [&](int l, int k, double2 v) {
-    const int a = l0 + 2 * l;
-    if (a < nlines) out[(size_t)a * n + k] = v.y;
-    if (a + 1 < nlines) out[(size_t)(a + 1) * n + k] = v.x;
-  });
+  for (int half = pass == FFT_Z ? 0 : 1;; ++half) {
+    line_fft(f);
+    if (half) break;
+    __syncthreads();
+#pragma unroll 4
+    for (int t = threadIdx.x; t < n << p.lsh; t += blockDim.x) {
+      const int l = t / p.by_n, k = t - l * n, line = min(f.l0 + l, f.nlines - 1);
+      const int kx = line / p.by_n, ky = line - kx * n;
+      const int my = 2 * ky < n ? ky : ky - n, mz = 2 * k < n ? k : k - n;
+      const int s = kx * kx + my * my + mz * mz;
+      double g;
+      if (kappa < 0.0)
+        g = c * __ldg(inv_s + s);
+      else
+        g = s == 0 ? c : c * (double)s / ((double)s + kappa);
+      double2 *v = f.nat + l * stride + k;
+      *v = make_double2(g * v->y, g * v->x);                   // exchanged: inverse
+    }
+    f.from_nat = true;
+    f.to_nat = false;
+    f.swap_out = true;
+    __syncthreads();
+  }
+  if (pass == FFT_X) {
+    __syncthreads();
+    for (int t = threadIdx.x; t < nh << p.lsh; t += blockDim.x) {
+      const int k = t >> p.lsh, l = t & ((1 << p.lsh) - 1), a = f.l0 + 2 * l;
+      const double2 zk = f.nat[l * stride + k], zr = f.nat[l * stride + (k ? n - k : 0)];
+      double2 *o = f.out + (size_t)k * f.nlines + a;
+      if (a < f.nlines) o[0] = make_double2(zk.x + zr.x, zk.y - zr.y);
+      if (a + 1 < f.nlines) o[1] = make_double2(zk.y + zr.y, zr.x - zk.x);
+    }
+  } else if (pass == FFT_XINV) {
+    __syncthreads();
+    double *x = static_cast<double *>(vout);
+    for (int t = threadIdx.x; t < n << p.lsh; t += blockDim.x) {
+      const int l = t / p.by_n, i = t - l * n, a = f.l0 + 2 * l;
+      const double2 v = f.nat[l * stride + i];
+      if (a < f.nlines) x[(size_t)a * n + i] = v.y;
+      if (a + 1 < f.nlines) x[(size_t)(a + 1) * n + i] = v.x;
+    }
+  }
 }
 
 // about the FP64 instructions of a butterfly, and its R - 1 twiddle products
@@ -643,6 +664,8 @@ bool line_plan(FftLine &p, int n) {
     p.by_r[s] = fast_div(p.r[s]);
     p.by_m[s] = fast_div(p.m[s]);
   }
+  p.by_n = fast_div(n);
+  p.by_nh = fast_div(n / 2 + 1);
   p.by_blocks = fast_div(n / p.r[p.ns - 1]);
   p.ls = (p.r[0] * (p.m[0] | 1)) | 1;
   // 8 lines: transposed writes of 128 bytes; 4 where two copies of the lines
@@ -677,11 +700,7 @@ const FftPlan *plan_of(int n) {
 // roots, 144 KB (once per process and device; setting it again changes nothing)
 void allow_large_shared() {
   const int most = 200 * 1024;
-  cudaFuncSetAttribute(k_fft_x, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  cudaFuncSetAttribute(k_fft_y<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  cudaFuncSetAttribute(k_fft_y<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  cudaFuncSetAttribute(k_fft_z_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  cudaFuncSetAttribute(k_fft_x_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(k_fft, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
 }  // namespace
@@ -698,14 +717,15 @@ void emd_fft2_multiply(int n, const double *in, double *out, double2 *wa, double
   const FftLine &p = plan_of(n)->line;
   const int per = 1 << p.lsh;
   const int bx = (n * n + 2 * per - 1) / (2 * per), by = (nh * n + per - 1) / per;
-  const size_t c16 = sizeof(double2);
-  const size_t one = (n + (size_t)per * p.ls) * c16, two = one + (size_t)per * (n | 1) * c16;
-  if (two > 49152) allow_large_shared();
-  const FastDiv by_n = fast_div(n), by_nh = fast_div(nh);
-  k_fft_x<<<bx, p.threads, two, st>>>(in, wa, p, nh, roots);
-  k_fft_y<false><<<by, p.threads, one, st>>>(wa, wb, p, nh, by_nh, roots);
-  // pass 1 leaves twice the spectrum
-  k_fft_z_factor<<<by, p.threads, two, st>>>(wb, wa, p, nh, by_n, 0.5 * c, kappa, inv_s, roots);
-  k_fft_y<true><<<by, p.threads, one, st>>>(wa, wb, p, nh, by_nh, roots);
-  k_fft_x_inv<<<bx, p.threads, two, st>>>(wb, out, p, nh, roots);
+  const size_t sm = (n + (size_t)per * (p.ls + (n | 1))) * sizeof(double2);
+  if (sm > 49152) allow_large_shared();
+  auto pass = [&](FftPass which, const void *src, void *dst, double scale) {
+    const int blocks = which == FFT_X || which == FFT_XINV ? bx : by;
+    k_fft<<<blocks, p.threads, sm, st>>>(which, src, dst, p, scale, kappa, inv_s, roots);
+  };
+  pass(FFT_X, in, wa, 0.0);
+  pass(FFT_Y, wa, wb, 0.0);
+  pass(FFT_Z, wb, wa, 0.5 * c);                   // the x pass leaves twice the spectrum
+  pass(FFT_YINV, wa, wb, 0.0);
+  pass(FFT_XINV, wb, out, 0.0);
 }
