@@ -39,8 +39,8 @@
 // butterflies have no twiddles to round, and sqrt(3) / 2 and sqrt(1/2) come with
 // their low parts, since the rounding of a constant that every line meets
 // scales the whole result (27^3: by 2.5e-16).
-#include <atomic>
 #include "emd_internal.cuh"
+#include "fft_plan.h"
 
 namespace {
 
@@ -352,51 +352,6 @@ template <> struct Dft<16> : DftAB<4, 4> {};
     case 16: CALL(16); break;                                                       \
   }
 
-// A line transform of n = r[0] r[1] .. r[ns-1] points, ns >= 2.  One step
-// turns a block of R m values x[j + m t] into R blocks of m: block k holds
-// w_{Rm}^{jk} sum_t w_R^{tk} x[j + m t] and is the transform of length m that
-// gives the frequencies k, k + R, ...; so a step reads and writes the same
-// places, and the last one leaves X[k_1 + r_1 (k_2 + r_2 (...))].  Line l's
-// first-step blocks start at l ls + k_1 (m_1 | 1) (odd strides: no conflicts).
-constexpr int kFftSteps = 4;
-// t / d for t d < 2^32 by one multiplication (an integer division is ~30
-// instructions, and a step of a small grid is only ~150)
-struct FastDiv {
-  unsigned mul, d;
-};
-__host__ __device__ __forceinline__ FastDiv fast_div(unsigned d) {
-  FastDiv f;
-  f.d = d;
-  f.mul = d > 1 ? 0xffffffffu / d + 1u : 0u;
-  return f;
-}
-__device__ __forceinline__ int operator/(int t, const FastDiv &f) {
-  return f.d == 1 ? t : (int)__umulhi((unsigned)t, f.mul);
-}
-struct FftLine {
-  int n, ns;              // grid edge and line length; steps
-  int r[kFftSteps];       // factors
-  int m[kFftSteps];       // block length after the step
-  FastDiv by_n, by_nh;    // nh: n / 2 + 1
-  FastDiv by_r[kFftSteps], by_m[kFftSteps], by_blocks;   // by_blocks: n / r[ns - 1]
-  int lsh;                // 2^lsh lines per CTA
-  int ls;                 // shared-memory stride of a line
-  int threads;            // per CTA
-};
-
-// block offset of frequency index kk = k_1 + r_1 (k_2 + ..) after `steps` steps
-__device__ __forceinline__ int block_at(const FftLine &p, int kk, int steps) {
-  if (steps == 1) return kk * (p.m[0] | 1);
-  int q = kk / p.by_r[0];
-  int off = (kk - q * p.r[0]) * (p.m[0] | 1);
-  for (int s = 1; s + 1 < steps; ++s) {
-    const int t = q / p.by_r[s];
-    off += (q - t * p.r[s]) * p.m[s];
-    q = t;
-  }
-  return off + q * p.m[steps - 1];
-}
-
 // The five passes are one kernel: the butterflies of 1 to 16 points are nearly
 // all of its code, and the first solve of a process waits until the code is on
 // the GPU (48^3: 0.7 ms for 0.5 MB; five kernels with a copy per transform were
@@ -618,84 +573,6 @@ k_fft(FftPass pass, const void *__restrict__ vin, void *__restrict__ vout,
   }
 }
 
-// about the FP64 instructions of a butterfly, and its R - 1 twiddle products
-int butterfly_cost(int R) {
-  static const int dft[17] = {0, 0, 4, 14, 16, 36, 44, 66, 64, 100, 92, 150, 108, 210, 156, 170, 160};
-  return dft[R] + 4 * (R - 1);
-}
-
-// the cheapest way to write n as 2 to 4 factors of at most 16, in ascending
-// order: a step costs its instructions times 64 cycles times the warps per
-// scheduler (at least one), and about 1500 cycles for its exchange
-void best_factors(FftLine &p, int nlines, int ns, int at, int left, int lo, int *r, double c,
-                  double &best) {
-  if (at == ns - 1) {
-    if (left > 16 || left < lo) return;
-    r[at] = left;
-    const double w = (double)nlines * (p.n / left) / 32.0 / 608.0;
-    c += (w > 1.0 ? w : 1.0) * (butterfly_cost(left) - 4 * (left - 1)) * 64.0;
-    if (c >= best) return;
-    best = c;
-    p.ns = ns;
-    for (int s = 0; s < ns; ++s) p.r[s] = r[s];
-    return;
-  }
-  for (int f = lo; f <= 16; ++f) {
-    if (left % f) continue;
-    const double w = (double)nlines * (p.n / f) / 32.0 / 608.0;
-    r[at] = f;
-    best_factors(p, nlines, ns, at + 1, left / f, f, r,
-                 c + 1500.0 + (w > 1.0 ? w : 1.0) * butterfly_cost(f) * 64.0, best);
-  }
-}
-
-// false: n is not a product of four factors of at most 16
-bool line_plan(FftLine &p, int n) {
-  const int nlines = n * (n / 2 + 1);
-  p.n = n;
-  p.ns = 0;
-  int r[kFftSteps];
-  double best = 1e300;
-  for (int ns = 2; ns <= kFftSteps; ++ns) best_factors(p, nlines, ns, 0, n, 1, r, 0.0, best);
-  if (!p.ns) return false;
-  int m = n;
-  for (int s = 0; s < p.ns; ++s) {
-    p.m[s] = m /= p.r[s];
-    p.by_r[s] = fast_div(p.r[s]);
-    p.by_m[s] = fast_div(p.m[s]);
-  }
-  p.by_n = fast_div(n);
-  p.by_nh = fast_div(n / 2 + 1);
-  p.by_blocks = fast_div(n / p.r[p.ns - 1]);
-  p.ls = (p.r[0] * (p.m[0] | 1)) | 1;
-  // 8 lines: transposed writes of 128 bytes; 4 where two copies of the lines
-  // and the roots pass 200 KB
-  p.lsh = (8 * (p.ls + n + 1) + n) * (int)sizeof(double2) <= 200 * 1024 ? 3 : 2;
-  const int most = (n / p.r[0]) << p.lsh;              // threads of the widest step
-  p.threads = most >= 256 ? 256 : (most + 31) / 32 * 32;
-  return true;
-}
-
-// The line plan of a grid, worked out once per size and kept for the life of
-// the process.
-struct FftPlan {
-  FftLine line;
-  bool ok;
-};
-constexpr int kFftMaxN = 1024;
-const FftPlan *plan_of(int n) {
-  static std::atomic<const FftPlan *> kept[kFftMaxN + 1];
-  if (n < 2 || n > kFftMaxN) return nullptr;
-  const FftPlan *p = kept[n].load();
-  if (!p) {
-    FftPlan *q = new FftPlan();
-    q->ok = line_plan(q->line, n);
-    if (kept[n].compare_exchange_strong(p, q)) p = q;
-    else delete q;
-  }
-  return p->ok ? p : nullptr;
-}
-
 // grids above ~190 points need more than 48 KB: 1024 takes 2 x 4 lines and the
 // roots, 144 KB (once per process and device; setting it again changes nothing)
 void allow_large_shared() {
@@ -705,7 +582,7 @@ void allow_large_shared() {
 
 }  // namespace
 
-bool emd_fft2_ok(int n) { return plan_of(n) != nullptr; }
+bool emd_fft2_ok(int n) { return fft_plan(n) != nullptr; }
 
 // out = the inverse transform of the spectral factor times the transform of
 // the real grid `in`.  in is read by the first pass only, so out may alias it;
@@ -714,10 +591,10 @@ void emd_fft2_multiply(int n, const double *in, double *out, double2 *wa, double
                        const double2 *roots, double c, double kappa, const double *inv_s,
                        cudaStream_t st) {
   const int nh = n / 2 + 1;                       // (n + 1) / 2 for odd n
-  const FftLine &p = plan_of(n)->line;
+  const FftLine &p = *fft_plan(n);
   const int per = 1 << p.lsh;
   const int bx = (n * n + 2 * per - 1) / (2 * per), by = (nh * n + per - 1) / per;
-  const size_t sm = (n + (size_t)per * (p.ls + (n | 1))) * sizeof(double2);
+  const size_t sm = fft_shared_bytes(p);
   if (sm > 49152) allow_large_shared();
   auto pass = [&](FftPass which, const void *src, void *dst, double scale) {
     const int blocks = which == FFT_X || which == FFT_XINV ? bx : by;
