@@ -573,11 +573,16 @@ k_fft(FftPass pass, const void *__restrict__ vin, void *__restrict__ vout,
   }
 }
 
-// grids above ~190 points need more than 48 KB: 1024 takes 2 x 4 lines and the
-// roots, 144 KB (once per process and device; setting it again changes nothing)
+// Grids above ~170 points need more than 48 KB of shared memory: asked for once
+// per device (again for devices past the 64th, which changes nothing).
 void allow_large_shared() {
-  const int most = 200 * 1024;
-  cudaFuncSetAttribute(k_fft, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  static std::atomic<bool> done[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return;     // the launch will fail and say so
+  if (dev < 64 && done[dev].load(std::memory_order_acquire)) return;
+  if (cudaFuncSetAttribute(k_fft, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kFftMaxShared) == cudaSuccess && dev < 64)
+    done[dev].store(true, std::memory_order_release);
 }
 
 }  // namespace
