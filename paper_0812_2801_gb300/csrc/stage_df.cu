@@ -67,19 +67,18 @@ template <int M> struct DFTile {
 // are read with four in flight); a separate instantiation keeps the
 // s-projector kernel's registers as they were.  IN / OUT: u_in / u_out as
 // split values (float4) instead of complex128; IN reads the split diagonal dv.
-// OUT = 2: complex128, and the split values over psi0 (dup): a point of psi0 is
+// OUT = 2: complex128, and the split values over psi0: a point of psi0 is
 // staged by the CTA that writes it, two planes before it writes it, and by no
 // other, so the next exponential's first stage reads split values without a
-// further orbital set.
+// further orbital set.  psi0 is therefore neither const nor restrict.
 template <int M, bool HCS, bool MP, bool IN, int OUT>
 __global__ void __launch_bounds__(256, 2)
-k_stage_df(const void *__restrict__ u_in, const double2 *__restrict__ psi0,
+k_stage_df(const void *__restrict__ u_in, double2 *psi0,
            void *__restrict__ u_out, const double *__restrict__ v_eff,
            const float2 *__restrict__ dv, const int4 *__restrict__ pt4d,
            const int *__restrict__ pt_J, const double *__restrict__ pt_p,
            const int4 *__restrict__ pt_rec, const double2 *__restrict__ hc, int n, int ntx,
-           int zc, int n_orb_pad, int n_proj, double a, int apply_only, float4 *dup,
-           DFWeights W) {
+           int zc, int n_orb_pad, int n_proj, double a, int apply_only, DFWeights W) {
   typedef DFTile<M> Z;
   constexpr int BO = Z::BO, NS = Z::NS, SW = Z::SW, NT = Z::NT;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -316,7 +315,7 @@ k_stage_df(const void *__restrict__ u_in, const double2 *__restrict__ psi0,
           const size_t o = boff + po * BO + j;
           if (OUT == 1) static_cast<float4 *>(u_out)[o] = df_split2(out);
           else static_cast<double2 *>(u_out)[o] = out;
-          if (OUT == 2) dup[o] = df_split2(out);
+          if (OUT == 2) reinterpret_cast<float4 *>(psi0)[o] = df_split2(out);
         }
       }
     }
@@ -373,10 +372,9 @@ void stage_df_tt(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
   const int smem = fixed + (HCS ? o.n_proj * Z::BO * (int)sizeof(float4) : 0);
   dim3 grid(ntx * nty, (o.n + zc - 1) / zc, o.n_blk);
   k_stage_df<M, HCS, MP, IN, OUT><<<grid, Z::NT, smem, st>>>(
-      a.u_in, (const double2 *)a.psi0, a.u_out, (const double *)a.v_eff,
+      a.u_in, (double2 *)const_cast<void *>(a.psi0), a.u_out, (const double *)a.v_eff,
       (const float2 *)a.v_diag, a.tab->pt4d, a.tab->pt_J, a.tab->pt_p, a.tab->pt_rec,
-      (const double2 *)a.hc, o.n, ntx, zc, o.n_orb_pad, o.n_proj, a.a, a.apply_only,
-      OUT == 2 ? (float4 *)a.psi0 : nullptr, W);
+      (const double2 *)a.hc, o.n, ntx, zc, o.n_orb_pad, o.n_proj, a.a, a.apply_only, W);
 }
 
 template <int M, bool MP>
