@@ -91,8 +91,8 @@ extern "C" {
 #define EMD_OPT_ZCHUNK       6  /* planes per z-chunk of the z-marching
                                    stage kernels (each CTA marches through
                                    one chunk and restages 2 * order / 2 halo
-                                   planes): 0 automatic (whole columns unless
-                                   that leaves SMs idle), else an integer
+                                   planes): 0 automatic (the split with the
+                                   smallest estimated time), else an integer
                                    1 .. 1024 (clamped to the grid)          */
 
 /* kernels that can be timed with EMD_OPT_PROFILE */

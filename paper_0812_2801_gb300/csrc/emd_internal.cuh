@@ -295,20 +295,10 @@ __device__ __forceinline__ void emd_block_sum(double (&v)[NV], double *smem) {
 // CTAs: NV <= 16 partial sums per CTA and one arrival counter per (projector,
 // orbital block); the counters are zero between launches.  Launches that use
 // one system's scratch are ordered (one stream at a time).
-constexpr int kGatherMaxCtas = 152 * 12 * 2;      // with a split, pairs x split stays below
 struct GatherScratch {
   double *part = nullptr;                         // [kGatherMaxCtas][16]
   int *arrived = nullptr;                         // [kGatherMaxCtas / 2]
 };
-// CTAs of 256 threads per (projector, orbital block): one when the pairs fill
-// the GPU, else 2, 4 or 8 that share the atom's entries.  Aims at 12 CTAs per
-// SM and at least one full round of the loop (1024 entries; about half of a
-// table's capacity, a cube around the sphere, is used) per CTA.
-inline int emd_gather_split(int pairs, int cap) {
-  int s = 1;
-  while (s < 8 && pairs * s < kGatherMaxCtas / 2 && cap / 2 >= 1024 * 2 * s) s *= 2;
-  return s;
-}
 
 // Sum of NV (a power of two <= 16) doubles per thread over the 256 threads of
 // `split` CTAs, in an order fixed by the launch shape.  FP64 adds are the cost
@@ -388,7 +378,7 @@ void emd_launch_wrap(const double *R, double *Rw, int n_atoms, double L,
                      cudaStream_t st);
 void emd_launch_tables(const GridInfo &g, const SpeciesDev &sp, int n_atoms,
                        TableSet &t, int *err, cudaStream_t st);
-// part: [n_atoms][EMD_SPLIT][3] scratch
+// part: [n_atoms][EMD_SPLIT_MAX][3] scratch
 void emd_launch_local_force(const GridInfo &g, const SpeciesDev &sp,
                             int n_atoms, const TableSet &t, const double *v_es_a,
                             const double *v_es_b, double *part, double *F,

@@ -6,6 +6,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <mutex>
+#include "launch_rules.h"
 #ifdef __CUDACC__
 #define EMD_HD __host__ __device__ __forceinline__
 #else
@@ -82,7 +83,7 @@ inline void best_factors(FftLine &p, int nlines, int ns, int at, int left, int l
   if (at == ns - 1) {
     if (left > 16 || left < lo) return;
     r[at] = left;
-    const double w = (double)nlines * (p.n / left) / 32.0 / 608.0;
+    const double w = (double)nlines * (p.n / left) / 32.0 / (4.0 * kSMs);
     c += (w > 1.0 ? w : 1.0) * (butterfly_cost(left) - 4 * (left - 1)) * 64.0;
     if (c >= best) return;
     best = c;
@@ -92,7 +93,7 @@ inline void best_factors(FftLine &p, int nlines, int ns, int at, int left, int l
   }
   for (int f = lo; f <= 16; ++f) {
     if (left % f) continue;
-    const double w = (double)nlines * (p.n / f) / 32.0 / 608.0;
+    const double w = (double)nlines * (p.n / f) / 32.0 / (4.0 * kSMs);
     r[at] = f;
     best_factors(p, nlines, ns, at + 1, left / f, f, r,
                  c + 1500.0 + (w > 1.0 ? w : 1.0) * butterfly_cost(f) * 64.0, best);

@@ -1510,26 +1510,9 @@ k_nl_force_df(const double2 *__restrict__ u, size_t n3, int n_blk,
 
 // ---- dispatch -------------------------------------------------------------
 
-// planes per z-chunk of a marching stage launch: the caller's choice, else the
-// split with the smallest estimated time.  A chunk restages and re-stencils 2M
-// halo planes and fills its ring (about two planes more); CTAs are dealt to 152
-// SMs in rounds, and one CTA alone on an SM runs at about 0.7 of the speed of
-// two.  (At least 304 CTAs or 16 planes per chunk, the earlier rule for one
-// 512-thread CTA per SM, gave 108 CTAs of 24 planes on 16 orbitals of 48^3.)
+// planes per z-chunk of a complex64 marching stage launch
 inline int stage_zchunk(const OrbLayout &o, int cols) {
-  if (o.zchunk > 0) return std::min(o.zchunk, o.n);
-  int best = o.n;
-  double cost = 0.0;
-  for (int nz = 1; nz <= std::max(1, o.n / 4); ++nz) {
-    const int zc = (o.n + nz - 1) / nz, ctas = cols * ((o.n + zc - 1) / zc);
-    const double load = (ctas + 151) / 152;
-    const double c = std::max(load, 1.4) * (zc + 2 * o.half_order + 2);
-    if (nz == 1 || c < 0.98 * cost) {
-      cost = c;
-      best = zc;
-    }
-  }
-  return best;
+  return o.zchunk > 0 ? std::min(o.zchunk, o.n) : emd_zchunk(o.n, o.half_order, cols, 1.0, 2);
 }
 
 template <typename T, int BO, int M>

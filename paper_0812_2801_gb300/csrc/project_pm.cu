@@ -506,7 +506,7 @@ void emd_launch_project_tile(const OrbLayout &o, const TableSet &t, int n_atoms,
   const int nt = (o.n + EMD_TILE - 1) / EMD_TILE;
   const int used = o.n_blk * o.bo;
   // 8 orbitals per block read 128-byte pieces; 4 where 8 leave SMs idle
-  if (n_atoms * ((used + 7) / 8) >= 2 * 152)
+  if (n_atoms * ((used + 7) / 8) >= 2 * kSMs)
     k_project_tile_reduce<8><<<dim3(n_atoms, (used + 7) / 8), 256, 0, st>>>(
         partial, t.at_ntiles, t.at_rows, nt * nt * nt, o.n_orb_pad, used, h3, h_kb, c,
         (float2 *)hc);

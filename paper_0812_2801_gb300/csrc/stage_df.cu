@@ -328,28 +328,6 @@ k_stage_df(const void *__restrict__ u_in, double2 *psi0,
   }
 }
 
-// Planes per z-chunk: the caller's choice, else the split with the smallest
-// estimated time.  A chunk of zc planes costs zc full planes and 2M halo
-// planes at about 0.3 of one (the z direction is 80 of 302 packed FP32
-// instructions); CTAs are dealt to 152 SMs in rounds, and one CTA alone on an
-// SM runs at about 0.7 of the speed of two.
-int df_zchunk(const OrbLayout &o, int cols) {
-  if (o.zchunk > 0) return o.zchunk < o.n ? o.zchunk : o.n;
-  int best = o.n;
-  double cost = 1e300;
-  for (int nz = 1; nz <= o.n / 4; ++nz) {
-    const int zc = (o.n + nz - 1) / nz;
-    const int ctas = cols * ((o.n + zc - 1) / zc);
-    const double load = (ctas + 151) / 152;
-    const double t = (load < 1.4 ? 1.4 : load) * (zc + 0.3 * 2 * o.half_order);
-    if (t < 0.98 * cost) {
-      cost = t;
-      best = zc;
-    }
-  }
-  return best;
-}
-
 template <int M, bool HCS, bool MP, bool IN, int OUT>
 void stage_df_tt(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
   typedef DFTile<M> Z;
@@ -361,7 +339,9 @@ void stage_df_tt(const OrbLayout &o, const StageArgs &a, cudaStream_t st) {
     attr_done = true;
   }
   const int ntx = (o.n + Z::TX - 1) / Z::TX, nty = (o.n + Z::TY - 1) / Z::TY;
-  const int zc = df_zchunk(o, ntx * nty * o.n_blk);
+  const int cols = ntx * nty * o.n_blk;
+  const int zc = o.zchunk > 0 ? std::min(o.zchunk, o.n)
+                              : emd_zchunk(o.n, o.half_order, cols, 0.3, 0);
   DFWeights W;
   for (int k = 0; k <= EMD_MAX_HALF_ORDER; ++k) W.num[k] = (float)o.num[k];
   const double sk = -1.0 / (2.0 * o.h * o.h * o.den);

@@ -919,7 +919,7 @@ void emd_launch_local_force(const GridInfo &g, const SpeciesDev &sp,
   // about 4 CTAs per SM: with 16 per atom, 8 atoms left each CTA several
   // rounds of rows (37 us on 48^3)
   const int nsplit = !t.gtab || n_atoms >= 38 ? EMD_SPLIT
-                                              : n_atoms <= 9 ? EMD_SPLIT_MAX : 608 / n_atoms;
+                                              : n_atoms <= 9 ? EMD_SPLIT_MAX : 4 * kSMs / n_atoms;
   dim3 grid(n_atoms, nsplit);
   if (t.gtab)
     k_local_force_rows<<<grid, 256, 0, st>>>(g.n, g.h, g.L, t.Rw, t.gtab, t.gtabd,
