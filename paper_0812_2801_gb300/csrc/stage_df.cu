@@ -26,7 +26,11 @@
 //    they skip the x/y shells and stage no x/y halo.
 //  * The z direction accumulates in a register line of 2M+1 outputs per
 //    point; three planes are unrolled, so the line moves by three slots once
-//    per three planes and each ring slot is a compile-time constant.
+//    per three planes and each ring slot is a compile-time constant.  Not at
+//    order 8 with several projectors per atom: there the two more slots and the
+//    epilogue in three copies crowd out the record loads (96^3, 9 projectors
+//    per atom, 32 orbitals: 3.89 ms per launch unrolled, 3.05 one plane at a
+//    time; order 6: 2.88 and 2.85, 4 projectors 1.46 either way).
 //  * Projector entries past a warp's longest list are skipped.
 // Each thread owns one orbital of one point of a 16 x 8 tile and marches
 // through z; 256 threads, 128 registers, two CTAs per SM, so that one CTA
@@ -81,6 +85,7 @@ k_stage_df(const void *__restrict__ u_in, double2 *psi0,
            int zc, int n_orb_pad, int n_proj, double a, int apply_only, DFWeights W) {
   typedef DFTile<M> Z;
   constexpr int BO = Z::BO, NS = Z::NS, SW = Z::SW, NT = Z::NT;
+  constexpr int PH = MP && M == 4 ? 1 : 3;     // planes unrolled
   extern __shared__ __align__(16) unsigned char smraw[];
   unsigned char *dfbase = smraw + 3 * Z::RSLOT;
   float4 *hcs = reinterpret_cast<float4 *>(dfbase + (IN ? 0 : 2 * Z::DSLOT));
@@ -175,11 +180,11 @@ k_stage_df(const void *__restrict__ u_in, double2 *psi0,
           df_split(__fma_rn(W.dvs, reinterpret_cast<const double *>(raw + Z::RU)[tid], W.dv0));
   };
 
-  // at phase ph of a group of three planes, [s + ph]: output plane zi - M + s,
+  // at phase ph of a group of PH planes, [s + ph]: output plane zi - M + s,
   // K as hi = (re, im), lo = (re, im)
-  float2 ah[NS + 2], al[NS + 2];
+  float2 ah[NS + PH - 1], al[NS + PH - 1];
 #pragma unroll
-  for (int s = 0; s < NS + 2; ++s) ah[s] = al[s] = make_float2(0.f, 0.f);
+  for (int s = 0; s < NS + PH - 1; ++s) ah[s] = al[s] = make_float2(0.f, 0.f);
   const int ci = ((yl + M) * SW + xl + M) * BO + j;        // centre, float4 index
   const int pt = yl * Z::TX + xl;                          // tile point index
   const char *hcj = reinterpret_cast<const char *>(hcs + j);
@@ -193,9 +198,9 @@ k_stage_df(const void *__restrict__ u_in, double2 *psi0,
     __syncthreads();
     convert(0);
   }
-  for (int zg = 0; zg < total; zg += 3) {
+  for (int zg = 0; zg < total; zg += PH) {
 #pragma unroll
-    for (int ph = 0; ph < 3; ++ph) {
+    for (int ph = 0; ph < PH; ++ph) {
       const int zi = zg + ph;
       if (zi >= total) break;
       // IN: planes zi and zi + 1 are in flight, wait for zi.  Else raw plane
@@ -208,7 +213,7 @@ k_stage_df(const void *__restrict__ u_in, double2 *psi0,
       __syncthreads();
       if (zi + 2 < total) issue(zi + 2);
       if (!IN && zi + 1 < total) convert(zi + 1);
-      const unsigned char *raw = smraw + ph * Z::RSLOT;
+      const unsigned char *raw = smraw + (PH == 3 ? ph : zi % 3) * Z::RSLOT;
       const unsigned char *base = IN ? raw : dfbase + (zi & 1) * Z::DSLOT;
       const float4 *P = reinterpret_cast<const float4 *>(base) + ci;
       const float4 c = P[0];
@@ -321,9 +326,9 @@ k_stage_df(const void *__restrict__ u_in, double2 *psi0,
     }
     // the next group's planes find output zi - M + s in slot s again
 #pragma unroll
-    for (int s = 0; s + 3 < NS + 2; ++s) {
-      ah[s] = ah[s + 3];
-      al[s] = al[s + 3];
+    for (int s = 0; s + PH < NS + PH - 1; ++s) {
+      ah[s] = ah[s + PH];
+      al[s] = al[s + PH];
     }
   }
 }
