@@ -351,8 +351,7 @@ void stage(emd_system *s, const void *u_in, const void *psi0, void *u_out,
 
 // Whether the double-float stage keeps its intermediate sets as split values.
 bool split_sets(const emd_system *s) {
-  return s->veff1s && s->o.stage_variant != 1 && (s->proj_atom_major || s->sp.nch > 1) &&
-         emd_stage_df_splits(s->o);
+  return s->veff1s && s->o.stage_variant != 1 && (s->proj_atom_major || s->sp.nch > 1);
 }
 
 // One exponential T4(-i tau H) psi0 -> out, H given by (set, veff).

@@ -502,7 +502,6 @@ struct OrbLayout {
 void emd_launch_stage(const OrbLayout &o, const StageArgs &a, cudaStream_t st);
 // stage_df.cu: the complex128, bo = 2 stage in double-float arithmetic
 void emd_launch_stage_df(const OrbLayout &o, const StageArgs &a, cudaStream_t st);
-bool emd_stage_df_splits(const OrbLayout &o);   // takes and writes split sets
 void emd_launch_project(const OrbLayout &o, const TableSet &t, int n_atoms,
                         const void *u, double h3, double h_kb, double2 *c,
                         void *hc, cudaStream_t st, bool u_split = false);

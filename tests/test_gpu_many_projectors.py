@@ -1,6 +1,6 @@
-"""The double-float FP64 stage with more than 1024 projectors, whose values then
-come from global memory and whose intermediate sets stay complex128, against
-the plain FP64 stage: 1125 projectors (125 atoms, l <= 2) and 1331 (one each).
+"""The double-float FP64 stage with more than 1024 projectors, whose h c then
+comes from global memory, against the plain FP64 stage: 1125 projectors (125
+atoms, l <= 2) and 1331 (one each).
 
 Tolerance: H u as against the oracle, 1e-12 of the largest value (48-bit
 products against 53-bit ones: ~4e-15 of the largest term, the kinetic diagonal's
