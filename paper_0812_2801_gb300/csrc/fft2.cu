@@ -370,7 +370,7 @@ template <> struct Dft<16> : DftAB<4, 4> {};
 //        2 are dropped.
 enum FftPass { FFT_X, FFT_Y, FFT_Z, FFT_YINV, FFT_XINV };
 
-// Shared memory of a CTA: the plan | roots | exchange array | lines in natural
+// Shared memory of a CTA: roots | exchange array | lines in natural
 // order (line l, element i at l (n | 1) + i).
 struct FftCta {
   FftPass pass;
